@@ -95,7 +95,9 @@ int qbvh_destroy(qbvh_handle h);
 /* Traversal mapping: 0 = one thread per particle (Alg. 1 as written);
  * 1 (default) = one warp per 32 consecutive Z-order particles walking the
  * tree together (same rope walk, warp-uniform control flow, each lane testing
- * its own sphere).  Both give the same list.  Takes effect at the next query. */
+ * its own sphere).  Exact lists with 32 particles per warp walk 32-wide boxes
+ * over the same Z-order instead of the binary tree.  Every mapping gives the
+ * same list.  Takes effect at the next query. */
 #define QBVH_OPT_TRAVERSAL 4
 /* Node storage: 0 (default) = 16-byte nodes with 10-bit quantized bounds
  * (Fig. 3b); 1 = 32-byte nodes with exact FP32 bounds (Fig. 3a); 2 = 32-byte
@@ -157,12 +159,9 @@ int qbvh_destroy(qbvh_handle h);
  * the two passes are faster; the autotuner decides per workload.  Takes
  * effect at the next call. */
 #define QBVH_OPT_FUSED_LJ 12
-/* Traversal work distribution for the one-particle-per-lane walk of exact
- * FP32 lists: 0 (default) = one warp of the grid per packet of 32 Z-order
- * particles; 1 = about as many warps as the GPU keeps resident, each taking
- * packets from a device-side queue until none are left (a warp that ends
- * early starts another packet instead of waiting for its block).  The list
- * is the same either way.  Takes effect at the next query. */
+/* 0 (default) or 1.  Selected a packet queue of an earlier traversal; the walk
+ * of 32-wide boxes that replaced it gives every packet its own warp, and the
+ * option is accepted without effect.  The list never depended on it. */
 #define QBVH_OPT_PERSISTENT 13
 
 int qbvh_set_option(qbvh_handle h, int option, int value);

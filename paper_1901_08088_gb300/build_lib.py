@@ -20,8 +20,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libqbvh.so")
-HEADERS = [os.path.join(CSRC, "qbvh_internal.cuh"), os.path.join(ROOT, "include", "qbvh.h")]
-SOURCES = ["api.cu", "build.cu", "sort.cu", "query.cu", "lj.cu", "noalloc.cu", "grid.cu", "small_build.cu"]
+HEADERS = [os.path.join(CSRC, "qbvh_internal.cuh"), os.path.join(CSRC, "query_common.cuh"), os.path.join(ROOT, "include", "qbvh.h")]
+SOURCES = ["api.cu", "build.cu", "sort.cu", "query.cu", "query_wide.cu", "lj.cu", "noalloc.cu", "grid.cu", "small_build.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fsigned-char",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

@@ -73,7 +73,7 @@ struct qbvh_ctx {
     int grid_tpp = 8;      // lanes per particle of the grid traversal
     int type_trees = 1;    // 1: one tree per (system, type); 0: one tree per system
     int fused_lj = 0;      // qbvh_query_lj_async: LJ terms inside the traversal where supported
-    int persistent = 0;    // traversal warps take packets from a queue
+    int persistent = 0;    // accepted and kept; the list does not depend on it (include/qbvh.h)
     int built_method = 0;
     const void *grid_pos = nullptr;   // positions recorded by a grid-method build
     int built_fmt = 0;     // node format of the last build
@@ -101,6 +101,7 @@ struct qbvh_ctx {
     DevBuf rows, counts;
     DevBuf cell_start, stype;
     DevBuf leaves64;
+    DevBuf boxes;
     DevBuf lj_partials, lj_blk_sys, lj_blk_first, lj_sys_blk;
     std::vector<int> lj_layout_off;   // offsets the LJ block tables were built for
     int lj_n_blocks = 0;
@@ -176,6 +177,15 @@ int upload_if_changed(qbvh_ctx *h, DevBuf &dst, std::vector<T> &cache, const std
     if (cudaMemcpyAsync(dst.p, src.data(), bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return QBVH_ERR_CUDA;
     cache = src;
     return QBVH_OK;
+}
+
+// the three levels of 32-wide nodes of the last build, one after the other
+void box_levels(const qbvh_ctx *h, float4 *level[3])
+{
+    const int nn = h->n > 0 ? h->n : 1;
+    level[0] = reinterpret_cast<float4 *>(h->boxes.p);
+    level[1] = level[0] + 4 * box_count(nn, 1);
+    level[2] = level[1] + 4 * box_count(nn, 2);
 }
 
 float round_up_f(double v)
@@ -277,6 +287,7 @@ int build_impl(qbvh_ctx *h, const void *pos_dev, int n, int n_sys, const int *of
     rc = rc ? rc : ensure(h, h->leaves, nn * sizeof(float4));
     if (f64) rc = rc ? rc : ensure(h, h->leaves64, nn * 4 * sizeof(double));
     rc = rc ? rc : ensure(h, h->leaf_q, nn * sizeof(uint2));
+    rc = rc ? rc : ensure(h, h->boxes, (box_count(nn, 1) + box_count(nn, 2) + box_count(nn, 3)) * 4 * sizeof(float4));
     rc = rc ? rc : ensure(h, h->range, nn * sizeof(int2));
     rc = rc ? rc : ensure(h, h->child, nn * sizeof(int2));
     rc = rc ? rc : ensure(h, h->par_int, nn * 4);
@@ -323,6 +334,7 @@ int build_impl(qbvh_ctx *h, const void *pos_dev, int n, int n_sys, const int *of
     a.nodes32 = h->node_fmt == 1 ? reinterpret_cast<float4 *>(h->nodes32.p) : nullptr;
     a.nodes21 = h->node_fmt == 2 ? reinterpret_cast<int4 *>(h->nodes21.p) : nullptr;
     a.leaves = reinterpret_cast<float4 *>(h->leaves.p);
+    box_levels(h, a.boxes);
     a.status = reinterpret_cast<DevStatus *>(h->status.p);
     a.sort_scratch = reinterpret_cast<unsigned *>(h->sort_scratch.p);
     a.sort_scratch_words = sort_scratch_bytes(n, passes) / sizeof(unsigned);
@@ -494,9 +506,8 @@ int query_enqueue(qbvh_ctx *h, const float *r_list_host, int cap, cudaStream_t s
     rc = rc ? rc : ensure(h, h->counts, (size_t)(h->n > 0 ? h->n : 1) * 4);
     if (rc) return rc;
     DevStatus *st = reinterpret_cast<DevStatus *>(h->status.p);
-    // the largest count and the traversal's packet queue start at zero (the
-    // error word keeps what the build found)
-    if (cudaMemsetAsync(&st->max_count, 0, 2 * sizeof(int), s) != cudaSuccess) return QBVH_ERR_CUDA;
+    // the largest count starts at zero (the error word keeps what the build found)
+    if (cudaMemsetAsync(&st->max_count, 0, sizeof(int), s) != cudaSuccess) return QBVH_ERR_CUDA;
     if (h->built_method == 1) {
         rc = grid_enqueue(h, q.r_list, q.rl2, cap, s);
         if (rc) return rc;
@@ -514,6 +525,11 @@ int query_enqueue(qbvh_ctx *h, const float *r_list_host, int cap, cudaStream_t s
     q.nodes21 = reinterpret_cast<const int4 *>(h->nodes21.p);
     q.node_fmt = h->built_fmt;
     q.leaves = reinterpret_cast<const float4 *>(h->leaves.p);
+    float4 *boxes[3];
+    box_levels(h, boxes);
+    q.box1 = boxes[0];
+    q.box2 = boxes[1];
+    q.box3 = boxes[2];
     q.leaf_q = reinterpret_cast<const uint2 *>(h->leaf_q.p);
     q.keys_sorted = h->keys[h->sorted].p;
     q.wide_keys = h->wide;
@@ -529,7 +545,6 @@ int query_enqueue(qbvh_ctx *h, const float *r_list_host, int cap, cudaStream_t s
     q.traversal = h->traversal;
     q.warp_particles = h->warp_particles;
     q.block = h->query_block;
-    q.persistent = h->persistent;
     q.f64 = h->f64 ? 1 : 0;
     q.leaves64 = h->f64 ? reinterpret_cast<const double4_32a *>(h->leaves64.p) : nullptr;
     q.L64 = h->L64;
@@ -627,7 +642,7 @@ int qbvh_destroy(qbvh_handle h)
                          &h->leaves, &h->leaf_q, &h->range, &h->child, &h->par_int, &h->par_leaf, &h->visit,
                          &h->seg, &h->acc, &h->seg_start, &h->frames, &h->sys, &h->sys_off, &h->status,
                          &h->rows, &h->counts, &h->cell_start, &h->stype, &h->lj_partials, &h->lj_blk_sys, &h->lj_blk_first,
-                         &h->lj_sys_blk, &h->leaves64};
+                         &h->lj_sys_blk, &h->leaves64, &h->boxes};
         for (DevBuf *b : all) release(*b);
         if (h->h_status) cudaFreeHost(h->h_status);
     }

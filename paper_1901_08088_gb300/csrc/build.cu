@@ -48,12 +48,15 @@ __device__ __forceinline__ unsigned acc_init(int f) { return (f >= 1 && f <= 3) 
 
 // Resets the per-tree accumulators, the status word and the radix-sort scratch
 // (histograms, tickets, look-back words) in one grid-stride pass.
-__global__ void prepare_kernel(unsigned *acc, int n_seg, DevStatus *status, unsigned *scratch, size_t words)
+__global__ void prepare_kernel(unsigned *acc, int n_seg, DevStatus *status, unsigned *scratch, size_t words,
+                               unsigned *boxes, size_t box_words)
 {
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t t = t0; t < (size_t)n_seg * 8; t += stride) acc[t] = acc_init((int)(t & 7));
     for (size_t t = t0; t < words; t += stride) scratch[t] = 0u;
+    // 32-wide nodes of levels 2 and 3: empty (lower corners +inf, upper 0)
+    for (size_t t = t0; t < box_words; t += stride) boxes[t] = (t & 7) < 3 ? 0x7F800000u : 0u;
     if (t0 == 0) {
         status->max_count = 0;
         status->err = 0u;
@@ -550,6 +553,56 @@ __device__ __forceinline__ void fit_climb(const BuildArgs &a, int node, int hi, 
     }
 }
 
+// The 32-wide node of the warp's leaves (level 1) and its shares of the block's
+// nodes of levels 2 and 3, kept in s_wide[level - 2][side][corner].  The
+// boundary that splits a node of a higher level, where it lies inside the warp's
+// run, is also the highest there, so each side of the warp's node belongs to one
+// side of the nodes above.  wb: bits of the lane's box (lo, hi), the empty box
+// past the last leaf.  Every lane calls this.
+template <bool WIDE>
+__device__ __forceinline__ void wide_boxes(const BuildArgs &a, int k, unsigned long long key, const unsigned (&wb)[6],
+                                           unsigned (*s_wide)[2][6])
+{
+    const int lane = threadIdx.x & 31;
+    const int k0 = k - lane;
+    if (k0 >= a.n) return;   // warp-uniform
+    const int tail = min(31, a.n - 1 - k0);
+    const int side = split_side(key, split_bit(__shfl_sync(0xFFFFFFFFu, key, 0), __shfl_sync(0xFFFFFFFFu, key, tail)));
+    unsigned v0 = 0u, v1 = 0u;   // lane f < 6: corner f of side 0 and of side 1
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+        const unsigned none = f < 3 ? 0x7F800000u : 0u;
+        const unsigned x0 = side == 0 ? wb[f] : none, x1 = side == 1 ? wb[f] : none;
+        const unsigned r0 = f < 3 ? __reduce_min_sync(0xFFFFFFFFu, x0) : __reduce_max_sync(0xFFFFFFFFu, x0);
+        const unsigned r1 = f < 3 ? __reduce_min_sync(0xFFFFFFFFu, x1) : __reduce_max_sync(0xFFFFFFFFu, x1);
+        if (lane == f) {
+            v0 = r0;
+            v1 = r1;
+        }
+    }
+    if (lane < 8) {
+        unsigned *box = reinterpret_cast<unsigned *>(a.boxes[0]) + 16 * (size_t)(k0 >> 5) + lane;
+        box[0] = v0;
+        box[8] = v1;
+    }
+    const int k1 = k0 + tail;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        const int sh = l == 0 ? 10 : 15;
+        const int f0 = (k0 >> sh) << sh, f1 = min(f0 + (1 << sh), a.n) - 1;
+        const int bit = split_bit(key_at<WIDE>(a.keys_sorted, f0), key_at<WIDE>(a.keys_sorted, f1));
+        const int s0 = split_side(key_at<WIDE>(a.keys_sorted, k0), bit);
+        const int s1 = split_side(key_at<WIDE>(a.keys_sorted, k1), bit);
+        if (lane < 3) {
+            atomicMin(&s_wide[l][s0][lane], v0);
+            atomicMin(&s_wide[l][s1][lane], v1);
+        } else if (lane < 6) {
+            atomicMax(&s_wide[l][s0][lane], v0);
+            atomicMax(&s_wide[l][s1][lane], v1);
+        }
+    }
+}
+
 // Resident blocks of the fit per SM (register cap).  The climb keeps blocks
 // alive, so more of them hide more of its latency: 8 blocks of 256 (32
 // registers, a few spilled) measured build 0.359 -> 0.348 ms at N = 2M
@@ -569,20 +622,25 @@ __global__ void __launch_bounds__(kBlock, Q21 ? 4 : QBVH_FIT_MIN_BLOCKS) fit_ker
     __shared__ float4 s_hi[F32 ? kBlock : 1];
     __shared__ float4 s_leaf[F32 ? kBlock : 1];     // FP32 box of leaf b0 + t: lower corner
     __shared__ float4 s_leafhi[F32 && F64 ? kBlock : 1];   // upper corner (double-precision data)
+    __shared__ unsigned s_wide[2][2][6];            // the block's share of its nodes of levels 2 and 3
     const int t = threadIdx.x;
     const int b0 = blockIdx.x * kBlock;
     const int b1 = min(b0 + kBlock, a.n) - 1;
     const int k = b0 + t;
     const bool live = k < a.n;
     s_done[t] = 0;
+    if (t < 24) s_wide[t / 12][(t / 6) & 1][t % 6] = t % 6 < 3 ? 0x7F800000u : 0u;
+    __syncthreads();
 
     // ---- leaf k and the words of internal node k --------------------------
     int hi = 0, leaf_up = -1, sg = 0;
     bool node_valid = false;
     int2 r = make_int2(0, -1), c = make_int2(0, 0);
     int up = -1, rope = QBVH_END;
+    unsigned wb[6] = {0x7F800000u, 0x7F800000u, 0x7F800000u, 0u, 0u, 0u};   // the leaf's box, lo and hi bits
+    unsigned long long key = 0ull;
     if (live) {
-        const unsigned long long key = key_at<WIDE>(a.keys_sorted, k);
+        key = key_at<WIDE>(a.keys_sorted, k);
         sg = seg_of_key<WIDE>(key, a.n_types);
         const SegInfo g = a.seg[sg];
         hi = g.start + g.count - 1;
@@ -608,6 +666,13 @@ __global__ void __launch_bounds__(kBlock, Q21 ? 4 : QBVH_FIT_MIN_BLOCKS) fit_ker
             const float4 p = __ldg(a.pos + orig);
             blo = bhi = mid = make_float3(p.x, p.y, p.z);
         }
+        // (adding +0 folds -0; the bits of valid coordinates order like the values)
+        wb[0] = __float_as_uint(blo.x + 0.f);
+        wb[1] = __float_as_uint(blo.y + 0.f);
+        wb[2] = __float_as_uint(blo.z + 0.f);
+        wb[3] = __float_as_uint(bhi.x + 0.f);
+        wb[4] = __float_as_uint(bhi.y + 0.f);
+        wb[5] = __float_as_uint(bhi.z + 0.f);
         const int leaf_rope = rope_after(a.range, k, hi);
         const unsigned tag = (unsigned)orig | ((leaf_rope >= 0 ? 1u : 0u) << 31);
         const float4 leaf = make_float4(mid.x, mid.y, mid.z, __uint_as_float(tag));
@@ -633,10 +698,18 @@ __global__ void __launch_bounds__(kBlock, Q21 ? 4 : QBVH_FIT_MIN_BLOCKS) fit_ker
             rope = rope_after(a.range, r.y, hi);
         }
     }
+    wide_boxes<WIDE>(a, k, key, wb, s_wide);
     const bool local = node_valid && r.x >= b0 && r.y <= b1;
     if (local && (k < r.x || k > r.y)) atomicOr(&a.status->err, QBVH_DEVERR_INTERNAL);
     bool pending = local && k >= r.x && k <= r.y;
     __syncthreads();
+    // the block's leaves lie in one node of level 2 (1024 leaves) and one of level 3
+    if (t < 24) {
+        const int l = t / 12, side = (t / 6) & 1, f = t % 6;
+        unsigned *w = reinterpret_cast<unsigned *>(a.boxes[1 + l]) + 16 * (size_t)(b0 >> (l == 0 ? 10 : 15)) + 8 * side + f;
+        if (f < 3) atomicMin(w, s_wide[l][side][f]);
+        else atomicMax(w, s_wide[l][side][f]);
+    }
 
     // ---- block part: rounds over the local nodes -----------------------------
     for (int round = 0; round < kBlock; ++round) {
@@ -700,8 +773,9 @@ void launch_build_prepare(const BuildArgs &a, cudaStream_t s)
     const size_t work = (size_t)a.n_seg * 8 > a.sort_scratch_words ? (size_t)a.n_seg * 8 : a.sort_scratch_words;
     int blocks = (int)((work + kBlock - 1) / kBlock);
     blocks = blocks < 1 ? 1 : (blocks > 1216 ? 1216 : blocks);
+    const size_t box_words = a.n > 0 ? 16 * (box_count(a.n, 2) + box_count(a.n, 3)) : 0;
     prepare_kernel<<<blocks, kBlock, 0, s>>>(a.seg_rootbits, a.n_seg, a.status, a.sort_scratch,
-                                             a.sort_scratch_words);
+                                             a.sort_scratch_words, reinterpret_cast<unsigned *>(a.boxes[1]), box_words);
 }
 
 void launch_morton(const BuildArgs &a, cudaStream_t s)

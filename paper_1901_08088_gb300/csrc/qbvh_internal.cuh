@@ -21,6 +21,7 @@
 //            hi64 high}, {left or first leaf, rope, 0, 0}; written only when
 //            that format is chosen
 //   leaves   float4 {x, y, z, original index | rope-is-internal<<31}
+//   boxes    4 x float4 per 32-wide node of levels 1 to 3 (box_count)
 // Node ids: k >= 0 internal node k, ~k (negative) leaf k, QBVH_END = INT32_MIN.
 #pragma once
 
@@ -320,7 +321,7 @@ struct SysInfo {
 
 struct DevStatus {
     int max_count;
-    unsigned next_packet;   // packet queue of the traversal (zeroed with max_count before each query)
+    unsigned pad0;
     unsigned err;
     unsigned pad;
 };
@@ -360,8 +361,30 @@ struct BuildArgs {
     float4 *nodes32;     // [2n] FP32 nodes or nullptr
     int4 *nodes21;       // [2n] 21-bit nodes or nullptr
     float4 *leaves;
+    float4 *boxes[3];    // 32-wide nodes of levels 1, 2, 3 (see box_count)
     DevStatus *status;
 };
+
+// 32-wide nodes over the sorted order (query_wide.cu): node k of level l bounds
+// leaves 32^l k .. 32^l (k + 1) - 1 with two boxes, of the leaves before and
+// after the highest boundary between Z-order cells (or trees) inside it, each
+// as {lo.x, lo.y, lo.z, hi.x}, {hi.y, hi.z, -, -}.  Number of nodes of a level:
+__host__ __device__ inline size_t box_count(int n, int level) { return ((size_t)n + (32u << (5 * (level - 1))) - 1) >> (5 * level); }
+
+// bit of the highest boundary inside a run of keys, from its first and last
+// (a run of equal keys has none: every key is then on side 0)
+template <typename K>
+__device__ __forceinline__ int split_bit(K first, K last)
+{
+    const unsigned long long x = (unsigned long long)(first ^ last);
+    return x ? 63 - __clzll((long long)x) : 63;
+}
+
+template <typename K>
+__device__ __forceinline__ int split_side(K key, int bit)
+{
+    return (int)(((unsigned long long)key >> bit) & 1ull);
+}
 
 void launch_build_prepare(const BuildArgs &a, cudaStream_t s);
 void launch_morton(const BuildArgs &a, cudaStream_t s);
@@ -397,6 +420,7 @@ struct QueryArgs {
     const int4 *nodes21;    // 21-bit node format (node_fmt == 2)
     int node_fmt;
     const float4 *leaves;
+    const float4 *box1, *box2, *box3;   // 32-wide nodes (box_count)
     const uint2 *leaf_q;   // quantized leaf boxes (candidate mode)
     const void *keys_sorted;
     bool wide_keys;
@@ -420,8 +444,6 @@ struct QueryArgs {
     float rl2_hi[64];
     double r2_64[64];
     int block;
-    int persistent;        // 1: resident warps take packets from a queue (one particle per lane)
-    int n_packets;         // packets of 32 / W particles
     int sparse_blocks;     // leading blocks that walk sparse trees one particle per warp
     float r_list[64];      // [a][b] list radius
     float rl2[64];         // fl(r * r)
@@ -438,6 +460,8 @@ struct QueryArgs {
 };
 
 void launch_query(const QueryArgs &a, cudaStream_t s);
+// exact lists with 32 particles per warp (query_wide.cu)
+void launch_query_wide(QueryArgs a, cudaStream_t s);
 
 // Traversal with the Lennard-Jones terms of the accepted pairs (a.lj = 1):
 // one system, one type, one particle per lane, exact lists of FP32 data.

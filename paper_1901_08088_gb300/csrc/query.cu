@@ -46,13 +46,12 @@
 // fl(dx * Linv) lies strictly inside (n - 1/2, n + 1/2): rint gives n, the
 // expression's own choice.  Hence a pair is accepted under exactly one image,
 // the one rint selects, with the same d2 -- and rows hold no duplicates.
-#include "qbvh_internal.cuh"
+#include "query_common.cuh"
 
 namespace qbvh {
 
 namespace {
 
-constexpr unsigned FULL = 0xFFFFFFFFu;
 struct Frame {
     float rx, ry, rz;   // R_lo
     float hx, hy, hz;   // bin width
@@ -128,62 +127,6 @@ __device__ __forceinline__ Node decode_21(const float4 a, const float4 b, const 
     return n;
 }
 
-// Read-only loads of tree words (nodes, leaves).  QBVH_TREE_EVICT_LAST = 1
-// marks them evict-last in L2, so that list writes streaming through L2 evict
-// them after everything else.  That paid while the list went out as 4-byte
-// stores (1.4 GB of DRAM writes per launch at N = 2M: query 1.92 -> 1.84 ms);
-// with whole-sector row writes (1.0 GB) plain loads are faster (10-bit nodes
-// 1.266 -> 1.240 ms, FP32 nodes 1.243 -> 1.237 ms), so it is off.
-// QBVH_NODE_V8 = 1 reads a 32-byte FP32 node with one 256-bit load (sm_100
-// and later) instead of two 128-bit ones (same speed, one instruction).
-#ifndef QBVH_TREE_EVICT_LAST
-#define QBVH_TREE_EVICT_LAST 0
-#endif
-#ifndef QBVH_NODE_V8
-#define QBVH_NODE_V8 1
-#endif
-__device__ __forceinline__ float4 tree_ld(const float4 *p)
-{
-#if QBVH_TREE_EVICT_LAST
-    unsigned long long pol;
-    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    float4 v;
-    asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
-        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(pol));
-    return v;
-#else
-    return __ldg(p);
-#endif
-}
-__device__ __forceinline__ int4 tree_ld(const int4 *p)
-{
-#if QBVH_TREE_EVICT_LAST
-    unsigned long long pol;
-    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
-    int4 v;
-    asm("ld.global.nc.L2::cache_hint.v4.s32 {%0, %1, %2, %3}, [%4], %5;"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
-    return v;
-#else
-    return __ldg(p);
-#endif
-}
-// both halves of a 32-byte FP32 node (32-byte aligned: node arrays come from
-// the allocator's 256-byte aligned blocks)
-__device__ __forceinline__ void node32_ld(const float4 *p, float4 &a, float4 &b)
-{
-#if QBVH_NODE_V8 && QBVH_TREE_EVICT_LAST
-    asm("ld.global.nc.L2::evict_last.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w) : "l"(p));
-#elif QBVH_NODE_V8
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w) : "l"(p));
-#else
-    a = tree_ld(p);
-    b = tree_ld(p + 1);
-#endif
-}
-
 // Raw words of a node, loaded ahead of use.
 struct Raw {
     int4 q;
@@ -252,22 +195,6 @@ __device__ __forceinline__ bool overlap_q(float px, float py, float pz, uint2 q,
     return overlap(px, py, pz, n, rs2);
 }
 
-// Store of one list entry.  QBVH_ROW_STORE: 0 = streaming (evict-first),
-// 1 = cache at L2 (.cg), 2 = default write-back.
-#ifndef QBVH_ROW_STORE
-#define QBVH_ROW_STORE 0
-#endif
-__device__ __forceinline__ void row_store(int *p, int v)
-{
-#if QBVH_ROW_STORE == 0
-    __stcs(p, v);
-#elif QBVH_ROW_STORE == 1
-    __stcg(p, v);
-#else
-    *p = v;
-#endif
-}
-
 // Row writer.  Entries past cap are counted, not written.  The list is never
 // read back by the traversal, so it is stored with the streaming (evict-first)
 // hint and does not push the tree out of L2.  (Gathering four entries into
@@ -296,14 +223,6 @@ __device__ __forceinline__ void row_store(int *p, int v)
 #ifndef QBVH_QUERY_SPLIT_IMAGES
 #define QBVH_QUERY_SPLIT_IMAGES 0
 #endif
-__device__ __forceinline__ void store_sector(int *dst, const int *ring)
-{
-    const int4 lo = make_int4(ring[0], ring[32], ring[64], ring[96]);
-    const int4 hi = make_int4(ring[128], ring[160], ring[192], ring[224]);
-    __stcs(reinterpret_cast<int4 *>(dst), lo);
-    __stcs(reinterpret_cast<int4 *>(dst) + 1, hi);
-}
-
 struct Row {
     int *row;
     int cap;
@@ -399,77 +318,6 @@ struct Row {
     }
 };
 
-struct Query {
-    float xi, yi, zi;     // own position
-    int self;             // own sorted index
-    int self_id;          // own original index
-    float nLx, nLy, nLz;  // image shift n L
-    float px, py, pz;     // image centre fl(x_i + n L)
-    float rl2;
-    float rl2_lo, rl2_hi; // double-precision data: band of the FP32 test around rl2
-    int pair;             // double-precision data: type pair of the current tree
-    // Lennard-Jones value of an image pair (fused option): per axis the
-    // difference fl(fl(xj - v1) - v2), the once-rounded x_j - x_i - n L
-    float vx1, vy1, vz1, vx2, vy2, vz2;
-};
-
-// d2 of the exact test (see the header comment) for leaf position q.
-// SHIFT = false is the zero image, where subtracting n L = 0 is the identity.
-template <bool SHIFT>
-__device__ __forceinline__ float exact_d2(const Query &c, const float4 q)
-{
-#if QBVH_F32X2
-    f32x2 dxy = f2_sub(f2_pack(q.x, q.y), f2_pack(c.xi, c.yi));
-    float dz = __fsub_rn(q.z, c.zi);
-    if (SHIFT) {
-        dxy = f2_sub(dxy, f2_pack(c.nLx, c.nLy));
-        dz = __fsub_rn(dz, c.nLz);
-    }
-    float sx, sy;
-    f2_unpack(f2_mul(dxy, dxy), sx, sy);
-    return __fadd_rn(__fadd_rn(sx, sy), __fmul_rn(dz, dz));
-#else
-    float dx = __fsub_rn(q.x, c.xi);
-    float dy = __fsub_rn(q.y, c.yi);
-    float dz = __fsub_rn(q.z, c.zi);
-    if (SHIFT) {
-        dx = __fsub_rn(dx, c.nLx);
-        dy = __fsub_rn(dy, c.nLy);
-        dz = __fsub_rn(dz, c.nLz);
-    }
-    return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-#endif
-}
-
-// Double-precision particle data (Sec. 2.2).  The list's decision is the
-// pinned FP64 expression
-//   dx = fl(xj - xi); dx = fl(dx - L rint(fl(dx Linv))), same for y, z,
-//   d2 = fl(fl(fl(dx^2) + fl(dy^2)) + fl(dz^2)) < fl(r^2),
-// taken under the walk's image without rint, as in FP32 (the argument in the
-// header comment holds with the FP64 unit roundoff).  The leaf words hold
-// the positions rounded to FP32, and the FP32 d2 of those decides whenever
-// it lies outside [rl2_lo, rl2_hi]: the host sets that band from a bound on
-// the difference of the two computations for pairs within the radius
-// (per component at most 2^-21 L, see qbvh_query), so it cannot change a
-// decision.  Inside the band the FP64 positions decide.
-template <bool SHIFT>
-__device__ __forceinline__ double exact_d2_64(const QueryArgs &A, const Query &c, int j)
-{
-    const double2 *pj = reinterpret_cast<const double2 *>(A.leaves64 + j);
-    const double2 *pi = reinterpret_cast<const double2 *>(A.leaves64 + c.self);
-    const double2 jxy = __ldg(pj), jz = __ldg(pj + 1), ixy = __ldg(pi), iz = __ldg(pi + 1);
-    double dx = __dsub_rn(jxy.x, ixy.x);
-    double dy = __dsub_rn(jxy.y, ixy.y);
-    double dz = __dsub_rn(jz.x, iz.x);
-    if (SHIFT) {
-        const double L = A.L64;
-        if (c.nLx != 0.f) dx = __dsub_rn(dx, c.nLx > 0.f ? L : -L);
-        if (c.nLy != 0.f) dy = __dsub_rn(dy, c.nLy > 0.f ? L : -L);
-        if (c.nLz != 0.f) dz = __dsub_rn(dz, c.nLz > 0.f ? L : -L);
-    }
-    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-}
-
 // The exact decision for leaf j under the current image (j != self).  SELF =
 // false leaves out the self test where the caller knows j cannot be the
 // particle itself.  (Under a non-zero image the particle's own copy is never
@@ -561,53 +409,6 @@ __device__ __forceinline__ void push_shared(Row &out, bool acc, int j, unsigned 
     out.count += __popc(m);
 }
 
-// 27-bit set of the periodic images whose padded search sphere overlaps the
-// root AABB of a tree (Sec. 2.3): bit 9 (nx+1) + 3 (ny+1) + (nz+1).
-__device__ __forceinline__ unsigned image_mask(float x, float y, float z, float L, const SegInfo &g, float rs2)
-{
-    float gap[3][3];
-    const float xs[3] = {x, y, z};
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const float p = (m == 1) ? xs[d] : __fadd_rn(xs[d], (m == 0) ? -L : L);
-            gap[d][m] = fmaxf(fmaxf(__fsub_rd(g.rlo[d], p), __fsub_rd(p, g.rhi[d])), 0.f);
-        }
-    }
-    unsigned mask = 0u;
-#pragma unroll
-    for (int mx = 0; mx < 3; ++mx)
-#pragma unroll
-        for (int my = 0; my < 3; ++my)
-#pragma unroll
-            for (int mz = 0; mz < 3; ++mz) {
-                const float d2 = __fmaf_rd(gap[0][mx], gap[0][mx],
-                                           __fmaf_rd(gap[1][my], gap[1][my], __fmul_rd(gap[2][mz], gap[2][mz])));
-                if (d2 <= rs2) mask |= 1u << (mx * 9 + my * 3 + mz);
-            }
-    return mask;
-}
-
-__device__ __forceinline__ void set_image(Query &c, int img, float L)
-{
-    const int nx = img / 9 - 1, ny = (img / 3) % 3 - 1, nz = img % 3 - 1;
-    c.nLx = nx == 0 ? 0.f : (nx > 0 ? L : -L);
-    c.nLy = ny == 0 ? 0.f : (ny > 0 ? L : -L);
-    c.nLz = nz == 0 ? 0.f : (nz > 0 ? L : -L);
-    c.px = nx == 0 ? c.xi : __fadd_rn(c.xi, c.nLx);
-    c.py = ny == 0 ? c.yi : __fadd_rn(c.yi, c.nLy);
-    c.pz = nz == 0 ? c.zi : __fadd_rn(c.zi, c.nLz);
-}
-
-template <bool WIDE>
-__device__ __forceinline__ int seg_of_sorted(const QueryArgs &a, int s)
-{
-    if (WIDE) return (int)(__ldg(reinterpret_cast<const unsigned long long *>(a.keys_sorted) + s) >> 30);
-    if (a.n_types > 1) return (int)(__ldg(reinterpret_cast<const unsigned *>(a.keys_sorted) + s) >> 30);
-    return 0;
-}
-
 // the frame of the 21-bit node format: same corner, 2^21 - 1 bins
 __device__ __forceinline__ Frame frame21_of(const SegInfo &g)
 {
@@ -639,13 +440,6 @@ __device__ __forceinline__ bool bad_node(int node, const SegInfo &g, int last)
 {
     const int idx = node ^ (node >> 31);   // node for internal ids, ~node for leaves
     return (unsigned)(idx - g.start) > (unsigned)(last - g.start);
-}
-
-// Largest row count: one atomic per warp, skipped when it cannot raise the maximum.
-__device__ __forceinline__ void warp_max_count(int my_count, DevStatus *status)
-{
-    const int m = __reduce_max_sync(FULL, my_count);
-    if ((threadIdx.x & 31) == 0 && m > 0 && m > __ldcg(&status->max_count)) atomicMax(&status->max_count, m);
 }
 
 // Last leaf of a bundle: the leaf before the rope target, or the tree's last leaf.
@@ -1524,37 +1318,6 @@ __device__ __forceinline__ void warp_walk(const QueryArgs &a, const Query &c, Ro
 #ifndef QBVH_REVERSE_BLOCKS
 #define QBVH_REVERSE_BLOCKS 1
 #endif
-// ---- sparse trees: one particle per warp ---------------------------------
-// A tree of few, widely spaced particles (the large spheres of a
-// size-asymmetric mixture) makes poor packets: 32 consecutive Z-order
-// particles then span much of the box, so a packet walk is 32 separate
-// walks run one after another on one warp, and the few such warps end long
-// after the rest (mixture L = 100: the 400 large particles' walks of the
-// small-particle tree took 1.5 ms against 0.55 ms for all small-small
-// pairs).  Tree `ta` of a single-system FP32 build of 2 to 4 types (32-bit
-// keys) is walked one particle per warp instead when it holds at most
-// QBVH_SPARSE_MAX particles and a packet of 32 spans more than twice its
-// largest list radius:
-// 32 L^3 / count > (2 r_max)^3.  The choice changes only which warp walks a
-// particle: the walk visits the same nodes and leaves in the same order, so
-// rows are the same either way.
-#ifndef QBVH_SPARSE_TREES
-#define QBVH_SPARSE_TREES 1
-#endif
-#ifndef QBVH_SPARSE_MAX
-#define QBVH_SPARSE_MAX 4096
-#endif
-__device__ __forceinline__ bool sparse_tree(const QueryArgs &a, int ta)
-{
-    const int count = a.seg[ta].count;
-    if (count == 0 || count > QBVH_SPARSE_MAX) return false;
-    const int T = a.n_types;
-    float r = 0.f;
-    for (int tb = 0; tb < T; ++tb) r = fmaxf(r, a.r_list[ta * T + tb]);
-    const float L = a.sys[0].L, d = 2.f * r;
-    return 32.f * L * L * L > (float)count * d * d * d;
-}
-
 // The leading a.sparse_blocks blocks: every particle of a sparse tree gets a
 // whole warp (W = 32: the lanes share the walk and split each bundle's
 // leaves), warps taking particles in a grid-stride loop.
@@ -1808,21 +1571,15 @@ __device__ __forceinline__ void warp_packet(const QueryArgs &a, int p)
     }
 }
 
-// Packets to warps.  Without PERSIST every warp of the grid walks one packet
-// (its index in the grid).  With PERSIST the grid holds about as many warps
-// as the GPU keeps resident, and each warp takes packets from a device
-// counter until they run out, so that a warp that ends early starts the next
-// packet instead of idling until its block's last warp ends.  The counter
-// only grows, so the loop ends.  With several types packets are taken from
-// the end of the sorted order first: the last trees (in a size-asymmetric
-// mixture the large particles, whose packets span wide regions and walk
-// longest) start first and overlap the rest instead of running alone at the
-// end (mixture L = 100: 2.05 -> 1.89 ms before sparse trees; one type gains
-// nothing from it, 1.84 -> 1.87 ms at N = 2M).
-template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool F64, bool LJ, bool PERSIST>
+// Packets to warps: every warp of the grid walks one packet (its index in the
+// grid).  With several types packets are taken from the end of the sorted order
+// first: the last trees (in a size-asymmetric mixture the large particles, whose
+// packets span wide regions and walk longest) start first and overlap the rest
+// instead of running alone at the end (mixture L = 100: 2.05 -> 1.89 ms before
+// sparse trees).
+template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool F64, bool LJ>
 __device__ __forceinline__ void warp_query(const QueryArgs &a)
 {
-    static_assert(!PERSIST || (!LJ && PHASE == 2), "packet queue: one launch, no per-block LJ records");
     constexpr bool SPARSE = QBVH_SPARSE_TREES && !WIDE && !ONE && !CAND && !F64 && PHASE == 2;
     int bid = (int)blockIdx.x, nblk = (int)gridDim.x;
     if (SPARSE && a.sparse_blocks > 0) {
@@ -1834,17 +1591,6 @@ __device__ __forceinline__ void warp_query(const QueryArgs &a)
         nblk -= a.sparse_blocks;
     }
     const bool rev = QBVH_REVERSE_BLOCKS && (ONE ? 1 : a.n_types) > 1;
-    if (PERSIST) {
-        const int lane = threadIdx.x & 31;
-        for (;;) {
-            int p = 0;
-            if (lane == 0) p = (int)atomicAdd(&a.status->next_packet, 1u);
-            p = __shfl_sync(FULL, p, 0);
-            if (p >= a.n_packets) break;
-            warp_packet<WIDE, CAND, FMT, W, ONE, PHASE, F64, LJ>(a, rev ? a.n_packets - 1 - p : p);
-        }
-        return;
-    }
     const int blk = rev ? nblk - 1 - bid : bid;
     warp_packet<WIDE, CAND, FMT, W, ONE, PHASE, F64, LJ>(a, (int)((blk * blockDim.x + threadIdx.x) >> 5));
 }
@@ -1852,59 +1598,17 @@ __device__ __forceinline__ void warp_query(const QueryArgs &a)
 template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool F64 = false>
 __global__ void QBVH_QUERY_BOUNDS query_warp_kernel(const __grid_constant__ QueryArgs a)
 {
-    warp_query<WIDE, CAND, FMT, W, ONE, PHASE, F64, false, false>(a);
-}
-
-// Double-precision data: the filtered walk of one particle per lane, with its
-// own register cap (the FP64 band decision needs more registers than the
-// FP32 walk's 32)
-#ifndef QBVH_QUERY_F64_MIN_BLOCKS
-#define QBVH_QUERY_F64_MIN_BLOCKS 6
-#endif
-template <int FMT, bool ONE>
-__global__ void __launch_bounds__(256, QBVH_QUERY_F64_MIN_BLOCKS) query_f64_kernel(const __grid_constant__ QueryArgs a)
-{
-    warp_query<false, false, FMT, 1, ONE, 2, true, false, false>(a);
-}
-
-// the one-particle-per-lane walk of exact FP32 lists with the packet queue
-template <bool WIDE, int FMT, bool ONE>
-__global__ void QBVH_QUERY_BOUNDS query_queue_kernel(const __grid_constant__ QueryArgs a)
-{
-    warp_query<WIDE, false, FMT, 1, ONE, 2, false, false, true>(a);
+    warp_query<WIDE, CAND, FMT, W, ONE, PHASE, F64, false>(a);
 }
 
 // the walk of one system of one type that also sums the LJ terms of its pairs
 template <int FMT>
 __global__ void __launch_bounds__(256, QBVH_QUERY_LJ_MIN_BLOCKS) query_warp_lj_kernel(const __grid_constant__ QueryArgs a)
 {
-    warp_query<false, false, FMT, 1, true, 2, false, true, false>(a);
+    warp_query<false, false, FMT, 1, true, 2, false, true>(a);
 }
 
 }  // namespace
-
-// SM count of the current device, looked up once per device (the value
-// only sizes the sparse-tree blocks: a stale or racing read costs speed, not
-// correctness; the table is written once per slot with the same value)
-static int sm_count_current()
-{
-    constexpr int kMaxDev = 64;
-    static int sms[kMaxDev] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
-        cudaGetLastError();
-        return 152;
-    }
-    int v = __atomic_load_n(&sms[dev], __ATOMIC_RELAXED);
-    if (v <= 0) {
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
-            cudaGetLastError();
-            v = 152;
-        }
-        __atomic_store_n(&sms[dev], v, __ATOMIC_RELAXED);
-    }
-    return v;
-}
 
 // leading blocks for sparse trees: about 8 warps per SM
 static int sparse_blocks_for(const QueryArgs &a)
@@ -1919,55 +1623,23 @@ static size_t stage_bytes(int block, bool stage, bool f64 = false)
     return stage ? (size_t)(block / 32) * (sizeof(BundleStage) + (f64 ? kStage * sizeof(int) : 0)) : 0;
 }
 
-// Blocks of `kernel` that one SM keeps resident at `block` threads and
-// `smem` bytes of dynamic shared memory (at least 1).
-static int resident_blocks(const void *kernel, int block, size_t smem)
-{
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, block, smem) != cudaSuccess || nb < 1) {
-        cudaGetLastError();
-        nb = 1;
-    }
-    return nb;
-}
-
-// The packet-queue walk: at most as many blocks as stay resident, plus the
-// sparse-tree blocks.
-template <int FMT, bool WIDE, bool ONE>
-static void launch_queue(QueryArgs a, cudaStream_t s, int grid, size_t sm)
-{
-    const void *k = reinterpret_cast<const void *>(&query_queue_kernel<WIDE, FMT, ONE>);
-    const int resident = sm_count_current() * resident_blocks(k, a.block, sm);
-    const int g = min(grid, resident) + a.sparse_blocks;
-    query_queue_kernel<WIDE, FMT, ONE><<<g, a.block, sm, s>>>(a);
-}
-
 template <int FMT, int W, int PHASE>
 static void launch_warp_phase(QueryArgs a, cudaStream_t s, int grid)
 {
     const int b = a.block;
     a.sparse_blocks = 0;
-    a.n_packets = grid * (b / 32);
     if (QBVH_SPARSE_TREES && PHASE == 2 && !a.wide_keys && !a.candidates && a.n_types > 1) {
         a.sparse_blocks = sparse_blocks_for(a);
         grid += a.sparse_blocks;
     }
     const size_t sm = stage_bytes(b, stage_on(W, a.candidates != 0, false));
-    if (PHASE == 2 && W == 1 && a.persistent && !a.candidates) {
-        if (a.wide_keys) launch_queue<FMT, true, false>(a, s, grid - a.sparse_blocks, sm);
-        else if (a.n_types == 1) launch_queue<FMT, false, true>(a, s, grid - a.sparse_blocks, sm);
-        else launch_queue<FMT, false, false>(a, s, grid - a.sparse_blocks, sm);
-        return;
-    }
-    if (a.wide_keys) {
-        if (a.candidates) query_warp_kernel<true, true, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
-        else query_warp_kernel<true, false, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
-    } else if (a.candidates) {
-        query_warp_kernel<false, true, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
-    } else if (a.n_types == 1) {
-        query_warp_kernel<false, false, FMT, W, true, PHASE><<<grid, b, sm, s>>>(a);
-    } else {
-        query_warp_kernel<false, false, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
+    if (a.candidates) {
+        if (a.wide_keys) query_warp_kernel<true, true, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
+        else query_warp_kernel<false, true, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
+    } else if constexpr (W > 1) {   // W = 1: query_wide.cu
+        if (a.wide_keys) query_warp_kernel<true, false, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
+        else if (a.n_types == 1) query_warp_kernel<false, false, FMT, W, true, PHASE><<<grid, b, sm, s>>>(a);
+        else query_warp_kernel<false, false, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
     }
 }
 
@@ -1999,18 +1671,6 @@ static void launch_thread(const QueryArgs &a, cudaStream_t s)
     }
 }
 
-// Double-precision particle data: the exact list of one system through the
-// warp walk with one particle per lane.
-template <int FMT>
-static void launch_f64(const QueryArgs &a, cudaStream_t s)
-{
-    const int b = a.block;
-    const int grid = (int)(((long long)((a.n + 31) / 32) * 32 + b - 1) / b);
-    const size_t sm = stage_bytes(b, stage_on(1, false, true), true);
-    if (a.n_types == 1) query_f64_kernel<FMT, true><<<grid, b, sm, s>>>(a);
-    else query_f64_kernel<FMT, false><<<grid, b, sm, s>>>(a);
-}
-
 int query_lj_blocks(int n, int block)
 {
     const long long threads = (long long)((n + 31) / 32) * 32;
@@ -2031,10 +1691,8 @@ void launch_query_lj(const QueryArgs &a, cudaStream_t s)
 void launch_query(const QueryArgs &a, cudaStream_t s)
 {
     if (a.n == 0) return;
-    if (a.f64) {
-        if (a.node_fmt == 0) launch_f64<0>(a, s);
-        else if (a.node_fmt == 1) launch_f64<1>(a, s);
-        else launch_f64<2>(a, s);
+    if (a.f64 || (a.traversal == 1 && a.warp_particles == 32 && !a.candidates)) {
+        launch_query_wide(a, s);
         return;
     }
     if (a.traversal == 0) {

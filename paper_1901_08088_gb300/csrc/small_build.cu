@@ -69,10 +69,12 @@ __global__ void __launch_bounds__(kSB, 1) small_build_kernel(const BuildArgs a)
     __shared__ unsigned s_acc[kMaxTrees * 8];   // count, min bits xyz, max bits xyz
     __shared__ SegInfo s_seg[kMaxTrees];
     __shared__ unsigned s_tot[256], s_dstart[256], s_wsum[8];
+    __shared__ unsigned s_wide[kItems + 1][2][6];   // 32-wide nodes of level 2 (1024 leaves), then level 3 (all)
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = a.n, T = a.n_types, TV = a.type_bound;
     const SysInfo sy = a.sys[0];
+    if (tid < (kItems + 1) * 12) s_wide[tid / 12][(tid / 6) & 1][tid % 6] = tid % 6 < 3 ? 0x7F800000u : 0u;
     if (tid < kMaxTrees * 8) s_acc[tid] = ((tid & 7) >= 1 && (tid & 7) <= 3) ? 0x7F800000u : 0u;
     if (tid == 0) {
         a.status->max_count = 0;
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(kSB, 1) small_build_kernel(const BuildArgs a)
     }
     __syncthreads();
 
-    // ---- leaves: words, 10-bit boxes ----------------------------------------
+    // ---- leaves: words, 10-bit boxes, 32-wide nodes ---------------------------
     {
         float4 pl[kItems];
 #pragma unroll
@@ -322,11 +324,52 @@ __global__ void __launch_bounds__(kSB, 1) small_build_kernel(const BuildArgs a)
 #pragma unroll
         for (int it = 0; it < kItems; ++it) {
             const int k = tid + it * kSB;
+            const float4 p = pl[it];
+            {
+                // as wide_boxes in build.cu: level 1 is the warp's run of 32 leaves
+                // (adding +0 folds -0; the bits of valid coordinates order like the values)
+                const int k0 = k - lane;
+                if (k0 < n) {
+                    const int k1 = min(k0 + 31, n - 1);
+                    const int side = split_side(kA[k], split_bit(kA[k0], kA[k1]));
+                    const float xs[3] = {p.x + 0.f, p.y + 0.f, p.z + 0.f};
+                    unsigned v0 = 0u, v1 = 0u;   // lane f < 6: corner f (lo, hi) of side 0 and of side 1
+#pragma unroll
+                    for (int f = 0; f < 6; ++f) {
+                        const unsigned none = f < 3 ? 0x7F800000u : 0u, bits = __float_as_uint(xs[f % 3]);
+                        const unsigned x0 = k < n && side == 0 ? bits : none, x1 = k < n && side == 1 ? bits : none;
+                        const unsigned r0 = f < 3 ? __reduce_min_sync(0xFFFFFFFFu, x0) : __reduce_max_sync(0xFFFFFFFFu, x0);
+                        const unsigned r1 = f < 3 ? __reduce_min_sync(0xFFFFFFFFu, x1) : __reduce_max_sync(0xFFFFFFFFu, x1);
+                        if (lane == f) {
+                            v0 = r0;
+                            v1 = r1;
+                        }
+                    }
+                    if (lane < 8) {
+                        unsigned *box = reinterpret_cast<unsigned *>(a.boxes[0]) + 16 * (k0 >> 5) + lane;
+                        box[0] = v0;
+                        box[8] = v1;
+                    }
+#pragma unroll
+                    for (int l = 0; l < 2; ++l) {
+                        const int f0 = l == 0 ? it * kSB : 0, f1 = l == 0 ? min(f0 + kSB, n) - 1 : n - 1;
+                        const int bit = split_bit(kA[f0], kA[f1]);
+                        unsigned(*node)[6] = s_wide[l == 0 ? it : kItems];
+                        const int s0 = split_side(kA[k0], bit), s1 = split_side(kA[k1], bit);
+                        if (lane < 3) {
+                            atomicMin(&node[s0][lane], v0);
+                            atomicMin(&node[s1][lane], v1);
+                        } else if (lane < 6) {
+                            atomicMax(&node[s0][lane], v0);
+                            atomicMax(&node[s1][lane], v1);
+                        }
+                    }
+                }
+            }
             if (k >= n) continue;
             const unsigned key = kA[k];
             const SegInfo &g = s_seg[T > 1 ? (int)(key >> 30) : 0];
             const int hi = g.start + g.count - 1;
-            const float4 p = pl[it];
             const int leaf_rope = rope_after(s_range, k, hi);
             const unsigned tag = (unsigned)vA[k] | ((leaf_rope >= 0 ? 1u : 0u) << 31);
             a.leaves[k] = make_float4(p.x, p.y, p.z, __uint_as_float(tag));
@@ -338,6 +381,14 @@ __global__ void __launch_bounds__(kSB, 1) small_build_kernel(const BuildArgs a)
         }
     }
     __syncthreads();
+    // levels 2 and 3 (one node: at most kSmallMax leaves)
+    if (tid < (kItems + 1) * 12) {
+        const int b = tid / 12, side = (tid / 6) & 1, f = tid % 6;
+        if (b == kItems)
+            reinterpret_cast<unsigned *>(a.boxes[2])[8 * side + f] = s_wide[b][side][f];
+        else if (b * kSB < n)
+            reinterpret_cast<unsigned *>(a.boxes[1])[16 * b + 8 * side + f] = s_wide[b][side][f];
+    }
 
     // ---- bottom-up fit: every leaf's thread climbs; at each internal node the
     // first child to arrive stops and the second computes the node (Sec. 2.1),
