@@ -510,15 +510,13 @@ __device__ __forceinline__ void sparse_walks(const QueryArgs &a)
     }
 }
 
-#ifndef QBVH_WIDE_BLOCKS
-#define QBVH_WIDE_BLOCKS 4
-#endif
-#ifndef QBVH_WIDE_BLOCKS4
-#define QBVH_WIDE_BLOCKS4 4
-#endif
-// ONE: a single tree (one system, one type)
+// ONE: a single tree (one system, one type).  Registers: 64 (32 warps per SM), or
+// 80 (24 warps) for one particle per lane with several trees, which spills under
+// 64: the L = 100 mixture 290 -> 258 us, 256 uneven systems 1413 -> 1275 us; one
+// tree 1027 -> 1013 us at N = 2,097,152 but 64 -> 67 us at 131,072 with r = 1.42.
+// 48 registers (40 warps) were slower everywhere (1027 -> 1140 us).
 template <bool ONE, bool F64, int W>
-__global__ void __launch_bounds__(256, W == 1 ? QBVH_WIDE_BLOCKS : QBVH_WIDE_BLOCKS4) wide_query_kernel(const __grid_constant__ QueryArgs a)
+__global__ void __launch_bounds__(256, W == 1 && !ONE ? 3 : 4) wide_query_kernel(const __grid_constant__ QueryArgs a)
 {
     constexpr int G = 32 / W;
     int blk = (int)blockIdx.x, nblk = (int)gridDim.x;
