@@ -18,7 +18,8 @@
 using namespace qbvh;
 
 namespace qbvh {
-int lj_particles_per_block();
+int lj_particles_per_block(int n, int tpp);
+bool lj_spread(int n);
 }
 
 // 1: one system of at most 3072 particles is built by one block (small_build.cu)
@@ -67,7 +68,8 @@ struct qbvh_ctx {
     int traversal = 1;
     int warp_particles = 32;
     int node_fmt = 0;      // 0: 10-bit quantized nodes (Fig. 3b), 1: FP32 nodes (Fig. 3a), 2: 21-bit nodes
-    int lj_tpp = 2;        // lanes per particle in the LJ pass
+    int lj_tpp = 2;        // lanes per particle in the LJ pass (few particles: lj_spread, unless the caller set them)
+    bool lj_tpp_set = false;
     int lj_zorder = 1;     // LJ pass walks particles in the tree's Z-order
     int method = 0;        // 0: quantized BVH, 1: uniform grid comparator
     int grid_tpp = 8;      // lanes per particle of the grid traversal
@@ -104,6 +106,7 @@ struct qbvh_ctx {
     DevBuf boxes;
     DevBuf lj_partials, lj_blk_sys, lj_blk_first, lj_sys_blk;
     std::vector<int> lj_layout_off;   // offsets the LJ block tables were built for
+    int lj_layout_particles = 0;      // and the particles per block
     int lj_n_blocks = 0;
     // uploads cached by content
     std::vector<SysInfo> up_sys;
@@ -677,6 +680,7 @@ int qbvh_set_option(qbvh_handle h, int option, int value)
     case QBVH_OPT_LJ_LANES:
         if (value < 1 || value > 32 || (value & (value - 1))) return QBVH_ERR_INVALID_ARG;
         h->lj_tpp = value;
+        h->lj_tpp_set = true;
         return QBVH_OK;
     case QBVH_OPT_LJ_ZORDER:
         if (value != 0 && value != 1) return QBVH_ERR_INVALID_ARG;
@@ -851,9 +855,10 @@ int qbvh_lj_forward(qbvh_handle h, const void *pos_dev, const float *eps_dev, co
     }
     DeviceGuard g(h->device);
     // block tables: every block covers particles of one system
-    const int B = lj_particles_per_block();
+    const int tpp = !h->lj_tpp_set && lj_spread(h->n) ? 0 : h->lj_tpp;
+    const int B = lj_particles_per_block(h->n, tpp);
     int rc = QBVH_OK;
-    if (h->lj_layout_off != h->off || h->lj_blk_sys.p == nullptr) {
+    if (h->lj_layout_off != h->off || h->lj_layout_particles != B || h->lj_blk_sys.p == nullptr) {
         std::vector<int> blk_sys, blk_first, sys_blk(h->n_sys + 1, 0);
         for (int k = 0; k < h->n_sys; ++k) {
             sys_blk[k] = (int)blk_sys.size();
@@ -878,6 +883,7 @@ int qbvh_lj_forward(qbvh_handle h, const void *pos_dev, const float *eps_dev, co
             cudaMemcpyAsync(h->lj_sys_blk.p, sys_blk.data(), sys_blk.size() * 4, cudaMemcpyHostToDevice, stream))
             return QBVH_ERR_CUDA;
         h->lj_layout_off = h->off;
+        h->lj_layout_particles = B;
     }
     const int np = 1 + 2 * T * T;
     rc = ensure(h, h->lj_partials, (size_t)(h->lj_n_blocks > 0 ? h->lj_n_blocks : 1) * np * 8);
@@ -894,7 +900,8 @@ int qbvh_lj_forward(qbvh_handle h, const void *pos_dev, const float *eps_dev, co
     a.blk_sys = reinterpret_cast<const int *>(h->lj_blk_sys.p);
     a.blk_first = reinterpret_cast<const int *>(h->lj_blk_first.p);
     a.n_blocks = h->lj_n_blocks;
-    a.tpp = h->lj_tpp;
+    a.particles = B;
+    a.tpp = tpp;
     a.eps = eps_dev;
     a.sig = sig_dev;
     a.e = e_dev;
