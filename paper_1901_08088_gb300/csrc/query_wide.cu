@@ -59,14 +59,17 @@
 // some lane's exact test could accept.
 //
 // Measured (query launch alone, rope walk before -> here, microseconds): N = 1000
-// 181 -> 20; 30,011 256 -> 58; 131,072 with r = 1.42 190 -> 64; 131,072 in double
-// precision 339 -> 129; 262,144 327 -> 167; the L = 100 mixture 576 -> 290; 256
-// uneven systems 1904 -> 1413; 2,097,152 1242 -> 1027.  With one particle per
-// lane it is bound by instruction issue (67% of the peak rate at N = 262,144,
-// 13.8 k warp instructions per packet) with 32 warps per SM, which its 64
-// registers and 28 KB of stages per block of 128 allow; two variants of the walk
-// (zero and other images) instead of one stalled on instruction fetch (nine
-// warps of every ten issue slots on the uneven systems).
+// 181 -> 20; 30,011 256 -> 58; 131,072 with r = 1.42 190 -> 65; 131,072 in double
+// precision 339 -> 130; 262,144 327 -> 159; the L = 100 mixture 576 -> 248; liquid/
+// vapor 1,000,000 646 -> 393; 32 x 65,536 1523 -> 1028; 256 uneven systems 1904 ->
+// 1230; 2,097,152 1242 -> 953.  Bound by instruction issue and shared memory
+// together (N = 262,144: 67% of the issue rate, 65% of the L1 data pipe); leaving
+// parts out at N = 2,097,152 put 39% of the time in writing the rows, 25% in the
+// group tests, 20% in the chunks' filter, 16% in boxes and set-up.  One code path
+// for every image matters: with a second one for the zero image the uneven systems
+// stalled on instruction fetch.
+#include <stddef.h>
+
 #include "query_common.cuh"
 
 namespace qbvh {
@@ -80,8 +83,9 @@ template <int W>
 struct __align__(16) WideStage {
     float x[64], y[64], z[64];        // survivors, slot = running index & 63
     int zid[64];                      // their Z-order indices, -1 for padding
-    int id[W == 1 ? 512 : 64];        // their original indices (W = 1: of the pool and the stage,
-                                      // reversed within a group: mask bit p belongs to slot p)
+    int id[W == 1 ? 512 : 64];        // their original indices (W = 1: of the pool and the stage, from
+                                      // the pool's first, reversed within a group: mask bit p
+                                      // belongs to slot p)
     unsigned mask[W == 1 ? kPool + 1 : 1][32];
     int ring[W == 1 ? 16 * 32 : 4];   // slot k of lane l at ring[32 k + l]
 };
@@ -103,7 +107,7 @@ struct OutRow {
 struct Walk {
     int tot;     // staged
     int tested;  // tested (a multiple of 32)
-    int grp;     // tested groups whose masks wait in the pool
+    int pool;    // first one whose group's masks wait in the pool
     int self;    // index of the lane's own particle among the survivors, or -1
 };
 
@@ -237,7 +241,7 @@ __device__ __forceinline__ unsigned group_mask(const QueryArgs &a, const Query &
             f2_unpack(f2_fma(dx, dx, f2_fma(dy, dy, f2_fma(dz, dz, r2))), t0, t1);
             m = __funnelshift_l(__float_as_uint(t0), m, 1);
             m = __funnelshift_l(__float_as_uint(t1), m, 1);
-            near = fminf(near, fminf(fabsf(t0), fabsf(t1)));
+            near = fminf(fminf(near, fabsf(t0)), fabsf(t1));
         }
     }
     if (__any_sync(FULL, !(near > band))) {
@@ -268,6 +272,45 @@ __device__ __forceinline__ unsigned group_mask(const QueryArgs &a, const Query &
     return m;
 }
 
+// One step of emit_pool: the highest set bit p of the lane's mask m takes its
+// survivor's index from the group's slots (group base g) to the ring at byte
+// offset off; an empty mask gives way to the next group's.  Without a set bit the
+// store goes to the free slot after the last entry (the load, four bytes before
+// the group's first slot, stays inside the stage).  Written out so that nothing
+// here is a branch: 15 instructions, where the compiled conditions took about 33
+// (N = 2,097,152: 1013 -> 953 us, 80 registers both).  What is left of it is shared
+// memory: 32 lanes read 32 places of the pool's indices, three to four
+// wavefronts.
+__device__ __forceinline__ void emit_step(unsigned &m, unsigned &off, unsigned &g, unsigned last, unsigned ring,
+                                          unsigned lane4)
+{
+    asm volatile(
+        "{\n"
+        ".reg .pred some, left, next;\n"
+        ".reg .u32 p, t, id;\n"
+        "bfind.u32 p, %0;\n"
+        "setp.ne.u32 some, %0, 0;\n"
+        "shl.b32 t, p, 2;\n"
+        "add.u32 t, t, %2;\n"
+        "ld.shared.u32 id, [t + %6];\n"
+        "add.u32 t, %4, %1;\n"
+        "st.shared.u32 [t], id;\n"
+        "@some add.u32 %1, %1, 128;\n"
+        "and.b32 %1, %1, 0x780;\n"
+        "shl.b32 t, 1, p;\n"          // 0 for an empty mask: p = -1 is clamped
+        "not.b32 t, t;\n"
+        "and.b32 %0, %0, t;\n"
+        "setp.ne.u32 left, %2, %3;\n"
+        "setp.eq.and.u32 next, %0, 0, left;\n"
+        "@next add.u32 %2, %2, 128;\n"
+        "@next add.u32 t, %2, %5;\n"
+        "@next ld.shared.u32 %0, [t + %7];\n"
+        "}\n"
+        : "+r"(m), "+r"(off), "+r"(g)
+        : "r"(last), "r"(ring), "r"(lane4), "n"(offsetof(WideStage<1>, id)), "n"(offsetof(WideStage<1>, mask))
+        : "memory");
+}
+
 // W = 1: the pool's survivors to the lanes' rows, each lane its own masks in
 // order, one entry per step; completed sectors leave the ring once per 8 steps
 // (at most 15 entries wait in its 16 slots).  A step either takes a bit or moves
@@ -275,37 +318,29 @@ __device__ __forceinline__ unsigned group_mask(const QueryArgs &a, const Query &
 __device__ __forceinline__ void emit_pool(WideStage<1> *st, OutRow &out, Walk &w)
 {
     const int lane = threadIdx.x & 31;
-    char *ring = reinterpret_cast<char *>(st->ring + lane);
-    int off = (out.count & 15) << 7;   // byte offset of the next free slot
-    int boff = (out.base & 15) << 7;
-    const unsigned *words = &st->mask[0][lane];
-    const unsigned *end = words + 32 * (w.grp - 1);
-    int slot = w.tested - 32 * w.grp;
-    unsigned m = *words;
+    const int groups = (w.tested - w.pool) >> 5;
+    const unsigned base = (unsigned)__cvta_generic_to_shared(st);
+    const unsigned ring = (unsigned)__cvta_generic_to_shared(st->ring + lane);
+    unsigned off = (out.count & 15) << 7;    // byte offset of the next free slot
+    unsigned boff = (out.base & 15) << 7;    // and of the first entry
+    unsigned g = base;
+    const unsigned last = base + 128 * (groups - 1);
+    unsigned m = st->mask[0][lane];
     do {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            // without a set bit the store goes to the free slot after the last entry
-            int p;
-            asm("bfind.u32 %0, %1;" : "=r"(p) : "r"(m));
-            p &= 31;
-            *reinterpret_cast<int *>(ring + off) = st->id[(slot & 511) + p];
-            if (m != 0u) off = (off + 128) & 0x780;
-            m &= ~(1u << p);
-            if (m == 0u && words != end) {
-                slot += 32;
-                words += 32;
-                m = *words;
-            }
-        }
+        for (int u = 0; u < 8; ++u) emit_step(m, off, g, last, ring, 4 * lane);
         if (((off - boff) & 0x780) >= 8 * 128) {
-            if (out.base + 8 <= out.cap) store_sector(out.row + out.base, reinterpret_cast<const int *>(ring + boff));
+            if (out.base + 8 <= out.cap) store_sector(out.row + out.base, st->ring + lane + (boff >> 2));
             out.base += 8;
             boff ^= 8 * 128;
         }
-    } while (__any_sync(FULL, m != 0u || words != end));
+    } while (__any_sync(FULL, m != 0u || g != last));
     out.count = out.base + (((off - boff) & 0x780) >> 7);
-    w.grp = 0;
+    // the staged survivors that wait for their group come first in the next pool
+    const int rest = st->id[32 * groups + lane];
+    __syncwarp();
+    st->id[lane] = rest;
+    w.pool = w.tested;
     __syncwarp();
 }
 
@@ -320,8 +355,7 @@ __device__ __forceinline__ void take_group(const QueryArgs &a, const Query &c, O
     if ((w.self >> 5) == (w.tested >> 5)) m &= ~(0x80000000u >> (w.self & 31));
     if (!part) m = 0u;
     if (W == 1) {
-        st->mask[w.grp][threadIdx.x & 31] = m;
-        ++w.grp;
+        st->mask[(w.tested - w.pool) >> 5][threadIdx.x & 31] = m;
     } else {
         constexpr int N = 32 / W;
         unsigned mine = (m << (N * wsub)) & ~(0xFFFFFFFFu >> N);
@@ -391,7 +425,7 @@ __device__ __forceinline__ void wide_walk(const QueryArgs &a, const Query &c, Ou
                         out.count += __popc(m);
                         continue;
                     }
-                    if (W == 1 && w.grp >= kPool) emit_pool(reinterpret_cast<WideStage<1> *>(st), out, w);
+                    if (W == 1 && w.tested - w.pool >= 32 * kPool) emit_pool(reinterpret_cast<WideStage<1> *>(st), out, w);
                     const bool surv = in && near_packet(p, Box{q.x, q.y, q.z, q.x, q.y, q.z}, rs2);
                     const unsigned S = __ballot_sync(FULL, surv);
                     const int r = w.tot + __popc(S & lanes_below());
@@ -401,7 +435,7 @@ __device__ __forceinline__ void wide_walk(const QueryArgs &a, const Query &c, Ou
                         st->y[k] = __fsub_rn(q.y, c.nLy);
                         st->z[k] = __fsub_rn(q.z, c.nLz);
                         st->zid[k] = j;
-                        st->id[W == 1 ? (r & 511) ^ 31 : k] = id;
+                        st->id[W == 1 ? (r - w.pool) ^ 31 : k] = id;
                     }
                     // the packet's own chunk hands every lane its own particle
                     // (a survivor wherever the lane walks this tree as its own)
@@ -439,7 +473,14 @@ __device__ __forceinline__ void walk_trees(const QueryArgs &a, Query &c, OutRow 
             c.rl2_hi = a.rl2_hi[pair];
             c.pair = pair;
         }
-        const unsigned mine = part ? image_mask(c.xi, c.yi, c.zi, L, g, rs2) : 0u;
+        // most packets see the tree under the zero image alone: no shift by L brings
+        // a lane's sphere to the root box on any axis (the rounding here, below
+        // 2^-22 L, is inside the 2^-19 L that rs adds to the radius)
+        const float rs = a.rs[pair];
+        const bool inner = c.xi - L + rs < g.rlo[0] && c.xi + L - rs > g.rhi[0] && c.yi - L + rs < g.rlo[1] &&
+                           c.yi + L - rs > g.rhi[1] && c.zi - L + rs < g.rlo[2] && c.zi + L - rs > g.rhi[2];
+        unsigned mine = part ? 1u << 13 : 0u;
+        if (!__all_sync(FULL, inner || !part)) mine = part ? image_mask(c.xi, c.yi, c.zi, L, g, rs2) : 0u;
         unsigned mask = __reduce_or_sync(FULL, mine);
         // band of the group test (header comment); every group is decided by the
         // pinned expression where r^2 is too small or too large for the bounds
@@ -454,7 +495,7 @@ __device__ __forceinline__ void walk_trees(const QueryArgs &a, Query &c, OutRow 
             const int img = __ffs(mask) - 1;
             mask &= mask - 1u;
             set_image(c, img, L);
-            wide_walk<F64, W>(a, c, out, st, w, first, last, (mine >> img) & 1u, part, side, a.rs[pair], rs2, band, L,
+            wide_walk<F64, W>(a, c, out, st, w, first, last, (mine >> img) & 1u, part, side, rs, rs2, band, L,
                               img == 13 && tb == ta ? own : -1, own_lane, wsub);
         }
         if (W < 32 && w.tot > w.tested) {
@@ -510,13 +551,13 @@ __device__ __forceinline__ void sparse_walks(const QueryArgs &a)
     }
 }
 
-// ONE: a single tree (one system, one type).  Registers: 64 (32 warps per SM), or
-// 80 (24 warps) for one particle per lane with several trees, which spills under
-// 64: the L = 100 mixture 290 -> 258 us, 256 uneven systems 1413 -> 1275 us; one
-// tree 1027 -> 1013 us at N = 2,097,152 but 64 -> 67 us at 131,072 with r = 1.42.
-// 48 registers (40 warps) were slower everywhere (1027 -> 1140 us).
+// ONE: a single tree (one system, one type).  Registers: 80 (24 warps per SM) for
+// one particle per lane, which spills under 64 (32 warps): N = 2,097,152 1039 -> 953
+// us, liquid/vapor 1,000,000 434 -> 393, the L = 100 mixture 290 -> 248; 48 registers
+// (40 warps) were slower still.  A single tree of double-precision data, whose FP64
+// decision is rare, is 133 us with 64 and 139 with 80 (N = 131,072).
 template <bool ONE, bool F64, int W>
-__global__ void __launch_bounds__(256, W == 1 && !ONE ? 3 : 4) wide_query_kernel(const __grid_constant__ QueryArgs a)
+__global__ void __launch_bounds__(256, W == 1 && !(ONE && F64) ? 3 : 4) wide_query_kernel(const __grid_constant__ QueryArgs a)
 {
     constexpr int G = 32 / W;
     int blk = (int)blockIdx.x, nblk = (int)gridDim.x;
@@ -579,7 +620,7 @@ __global__ void __launch_bounds__(256, W == 1 && !ONE ? 3 : 4) wide_query_kernel
                            wsub);
     }
     if (W == 1) {
-        if (w.grp > 0) emit_pool(reinterpret_cast<WideStage<1> *>(st), out, w);
+        if (w.tested > w.pool) emit_pool(reinterpret_cast<WideStage<1> *>(st), out, w);
         // the last, partial sectors
         const int end = active && !elsewhere ? min(out.count, out.cap) : 0;
         for (int k = out.base; k < end; ++k) row_store(out.row + k, st->ring[32 * (k & 15) + lane]);
