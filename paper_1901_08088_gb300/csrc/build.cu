@@ -28,7 +28,7 @@ namespace {
 
 constexpr int kBlock = 256;
 constexpr int kLocalSegs = 64;
-constexpr int kMortonItems = 8;   // particles per thread of the Morton pass
+constexpr int kMortonItems = 8;   // most particles per thread of the Morton pass
 
 __device__ __forceinline__ int sys_of(const int *off, int n_sys, int i)
 {
@@ -51,6 +51,7 @@ __device__ __forceinline__ unsigned acc_init(int f) { return (f >= 1 && f <= 3) 
 __global__ void prepare_kernel(unsigned *acc, int n_seg, DevStatus *status, unsigned *scratch, size_t words,
                                unsigned *boxes, size_t box_words)
 {
+    pdl_begin();
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t t = t0; t < (size_t)n_seg * 8; t += stride) acc[t] = acc_init((int)(t & 7));
@@ -81,8 +82,9 @@ __device__ __forceinline__ void read_pos64(const BuildArgs &a, int idx, float3 &
 }
 
 template <bool WIDE, bool F64>
-__global__ void __launch_bounds__(kBlock) morton_kernel(const BuildArgs a, unsigned *acc)
+__global__ void __launch_bounds__(kBlock) morton_kernel(const BuildArgs a, unsigned *acc, int items)
 {
+    pdl_begin();
     __shared__ unsigned s_acc[kLocalSegs * 8];
     __shared__ unsigned s_hist[8 * 256];
     __shared__ int s_seg0, s_span;
@@ -91,8 +93,8 @@ __global__ void __launch_bounds__(kBlock) morton_kernel(const BuildArgs a, unsig
     const int npass = a.sort_passes;
     for (int t = threadIdx.x; t < npass * 256; t += kBlock) s_hist[t] = 0u;
     if (threadIdx.x == 0) {
-        int first = blockIdx.x * kBlock * kMortonItems;
-        int last = min(first + kBlock * kMortonItems, a.n) - 1;
+        int first = blockIdx.x * kBlock * items;
+        int last = min(first + kBlock * items, a.n) - 1;
         int k0 = a.n_sys > 1 ? sys_of(a.sys_off, a.n_sys, first) : 0;
         int k1 = a.n_sys > 1 ? sys_of(a.sys_off, a.n_sys, last) : 0;
         s_seg0 = k0 * T;
@@ -102,11 +104,16 @@ __global__ void __launch_bounds__(kBlock) morton_kernel(const BuildArgs a, unsig
     __syncthreads();
     const bool local = s_span <= kLocalSegs;
 
-    // kMortonItems particles per thread, in kBlock-wide strides: the block's
+    // `items` particles per thread, in kBlock-wide strides: the block's
     // histograms and tree accumulators go to global memory once per
-    // kBlock * kMortonItems particles
-    for (int it = 0; it < kMortonItems; ++it) {
-    const int i = (blockIdx.x * kMortonItems + it) * kBlock + threadIdx.x;
+    // kBlock * items particles.  The next particle is loaded one step ahead.
+    float4 pnext = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!F64 && (int)(blockIdx.x * items * kBlock + threadIdx.x) < a.n)
+        pnext = __ldg(a.pos + blockIdx.x * items * kBlock + threadIdx.x);
+    for (int it = 0; it < items; ++it) {
+    const int i = (blockIdx.x * items + it) * kBlock + threadIdx.x;
+    const float4 pin = pnext;
+    if (!F64 && it + 1 < items && i + kBlock < a.n) pnext = __ldg(a.pos + i + kBlock);
     if (i < a.n) {
         // fresh arrival counters and parent links for the fit (a missing link
         // ends a walk instead of sending it to an arbitrary index)
@@ -135,7 +142,7 @@ __global__ void __launch_bounds__(kBlock) morton_kernel(const BuildArgs a, unsig
             p = make_float4(lo.x, lo.y, lo.z, 0.f);
             ph = hi;
         } else {
-            p = __ldg(a.pos + i);
+            p = pin;
             type = __float_as_int(p.w);
             if (type < 0 || type >= TV) {
                 err |= QBVH_DEVERR_BAD_TYPE;
@@ -220,6 +227,7 @@ __global__ void __launch_bounds__(kBlock) morton_kernel(const BuildArgs a, unsig
 // One block: exclusive scan of the tree counts, tree records and frames.
 __global__ void __launch_bounds__(1024) seg_scan_kernel(const BuildArgs a, const unsigned *acc)
 {
+    pdl_begin();
     __shared__ int s_warp[32];
     __shared__ int s_carry;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -311,6 +319,7 @@ __device__ __forceinline__ int delta(const void *keys, int i, unsigned ci, int j
 template <bool WIDE>
 __global__ void __launch_bounds__(kBlock) karras_kernel(const BuildArgs a)
 {
+    pdl_begin();
     const int i = blockIdx.x * kBlock + threadIdx.x;
     if (i >= a.n) return;
     const unsigned long long key = key_at<WIDE>(a.keys_sorted, i);
@@ -350,6 +359,15 @@ __global__ void __launch_bounds__(kBlock) karras_kernel(const BuildArgs a)
     if (left >= 0) a.par_int[left] = i; else a.par_leaf[~left] = i;
     if (right >= 0) a.par_int[right] = i; else a.par_leaf[~right] = i;
     if (i == lo) a.par_int[i] = -1;   // node lo of a tree is its root
+    // the rope (rope_after): node last + 1 starts there when its range runs upwards,
+    // which its neighbours' keys tell without waiting for that node
+    int rope = QBVH_END;
+    if (last < hi) {
+        const int k = last + 1;
+        const unsigned ck = (unsigned)key_at<WIDE>(K, k) & QBVH_QMASK;
+        rope = k < hi && delta<WIDE>(K, k, ck, k + 1, lo, hi) > delta<WIDE>(K, k, ck, k - 1, lo, hi) ? k : ~k;
+    }
+    a.nodes[i].w = rope;
 }
 
 // 21-bit fields, three per 64-bit word (x << 42 | y << 21 | z)
@@ -503,7 +521,7 @@ __device__ __forceinline__ void fit_climb(const BuildArgs &a, int node, int hi, 
         const int2 r = a.range[node];
         const int2 c = a.child[node];
         const int up = a.par_int[node];
-        const int rope = rope_after(a.range, r.y, hi);
+        const int rope = __ldcg(&a.nodes[node].w);   // from the hierarchy pass
         // release publishes this child's bounds, acquire makes the sibling's
         // bounds visible to the thread that continues upward
         if (arrive_acq_rel(a.visit + node) == 0) return;   // sibling not done yet
@@ -613,6 +631,7 @@ __device__ __forceinline__ void wide_boxes(const BuildArgs &a, int k, unsigned l
 template <bool WIDE, bool F32, bool F64, bool Q21>
 __global__ void __launch_bounds__(kBlock, Q21 ? 4 : QBVH_FIT_MIN_BLOCKS) fit_kernel(const BuildArgs a)
 {
+    pdl_begin();
     __shared__ ulonglong2 s_q21[Q21 ? kBlock : 1];  // 21-bit box of internal node b0 + t
     __shared__ ulonglong2 s_lq21[Q21 ? kBlock : 1]; // 21-bit box of leaf b0 + t
     __shared__ int s_done[kBlock];                  // local internal node b0 + t settled
@@ -695,7 +714,7 @@ __global__ void __launch_bounds__(kBlock, Q21 ? 4 : QBVH_FIT_MIN_BLOCKS) fit_ker
             r = a.range[k];
             c = a.child[k];
             up = a.par_int[k];
-            rope = rope_after(a.range, r.y, hi);
+            rope = a.nodes[k].w;   // from the hierarchy pass; nobody else writes node k before this thread
         }
     }
     wide_boxes<WIDE>(a, k, key, wb, s_wide);
@@ -781,26 +800,29 @@ void launch_build_prepare(const BuildArgs &a, cudaStream_t s)
 void launch_morton(const BuildArgs &a, cudaStream_t s)
 {
     if (a.n == 0) return;
-    if (a.wide_keys)
-        morton_kernel<true, false><<<blocks_for(a.n, kBlock * kMortonItems), kBlock, 0, s>>>(a, a.seg_rootbits);
-    else if (a.pos64)
-        morton_kernel<false, true><<<blocks_for(a.n, kBlock * kMortonItems), kBlock, 0, s>>>(a, a.seg_rootbits);
-    else
-        morton_kernel<false, false><<<blocks_for(a.n, kBlock * kMortonItems), kBlock, 0, s>>>(a, a.seg_rootbits);
+    // few particles per thread while the grid has less than two blocks per SM: the
+    // items of a thread follow one another (N = 30,011: 15 blocks of 8 items each
+    // took 10 us), many where a block's histograms are worth sharing
+    int items = kMortonItems;
+    while (items > 1 && blocks_for(a.n, kBlock * items) < 304) items >>= 1;
+    const int g = blocks_for(a.n, kBlock * items);
+    if (a.wide_keys) launch_pdl(morton_kernel<true, false>, g, kBlock, 0, s, a, a.seg_rootbits, items);
+    else if (a.pos64) launch_pdl(morton_kernel<false, true>, g, kBlock, 0, s, a, a.seg_rootbits, items);
+    else launch_pdl(morton_kernel<false, false>, g, kBlock, 0, s, a, a.seg_rootbits, items);
 }
 
 void launch_seg_scan(const BuildArgs &a, cudaStream_t s)
 {
-    seg_scan_kernel<<<1, 1024, 0, s>>>(a, a.seg_rootbits);
+    launch_pdl(seg_scan_kernel, 1, 1024, 0, s, a, (const unsigned *)a.seg_rootbits);
 }
 
 void launch_karras(const BuildArgs &a, cudaStream_t s)
 {
     if (a.n == 0) return;
     if (a.wide_keys)
-        karras_kernel<true><<<blocks_for(a.n, kBlock), kBlock, 0, s>>>(a);
+        launch_pdl(karras_kernel<true>, blocks_for(a.n, kBlock), kBlock, 0, s, a);
     else
-        karras_kernel<false><<<blocks_for(a.n, kBlock), kBlock, 0, s>>>(a);
+        launch_pdl(karras_kernel<false>, blocks_for(a.n, kBlock), kBlock, 0, s, a);
 }
 
 void launch_fit(const BuildArgs &a, cudaStream_t s)
@@ -808,17 +830,17 @@ void launch_fit(const BuildArgs &a, cudaStream_t s)
     if (a.n == 0) return;
     const int g = blocks_for(a.n, kBlock);
     if (a.wide_keys) {
-        if (a.nodes32) fit_kernel<true, true, false, false><<<g, kBlock, 0, s>>>(a);
-        else if (a.nodes21) fit_kernel<true, false, false, true><<<g, kBlock, 0, s>>>(a);
-        else fit_kernel<true, false, false, false><<<g, kBlock, 0, s>>>(a);
+        if (a.nodes32) launch_pdl(fit_kernel<true, true, false, false>, g, kBlock, 0, s, a);
+        else if (a.nodes21) launch_pdl(fit_kernel<true, false, false, true>, g, kBlock, 0, s, a);
+        else launch_pdl(fit_kernel<true, false, false, false>, g, kBlock, 0, s, a);
     } else if (a.pos64) {
-        if (a.nodes32) fit_kernel<false, true, true, false><<<g, kBlock, 0, s>>>(a);
-        else if (a.nodes21) fit_kernel<false, false, true, true><<<g, kBlock, 0, s>>>(a);
-        else fit_kernel<false, false, true, false><<<g, kBlock, 0, s>>>(a);
+        if (a.nodes32) launch_pdl(fit_kernel<false, true, true, false>, g, kBlock, 0, s, a);
+        else if (a.nodes21) launch_pdl(fit_kernel<false, false, true, true>, g, kBlock, 0, s, a);
+        else launch_pdl(fit_kernel<false, false, true, false>, g, kBlock, 0, s, a);
     } else {
-        if (a.nodes32) fit_kernel<false, true, false, false><<<g, kBlock, 0, s>>>(a);
-        else if (a.nodes21) fit_kernel<false, false, false, true><<<g, kBlock, 0, s>>>(a);
-        else fit_kernel<false, false, false, false><<<g, kBlock, 0, s>>>(a);
+        if (a.nodes32) launch_pdl(fit_kernel<false, true, false, false>, g, kBlock, 0, s, a);
+        else if (a.nodes21) launch_pdl(fit_kernel<false, false, false, true>, g, kBlock, 0, s, a);
+        else launch_pdl(fit_kernel<false, false, false, false>, g, kBlock, 0, s, a);
     }
 }
 

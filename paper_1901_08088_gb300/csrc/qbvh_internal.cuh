@@ -383,6 +383,35 @@ struct BuildArgs {
 // as {lo.x, lo.y, lo.z, hi.x}, {hi.y, hi.z, -, -}.  Number of nodes of a level:
 __host__ __device__ inline size_t box_count(int n, int level) { return ((size_t)n + (32u << (5 * (level - 1))) - 1) >> (5 * level); }
 
+// Build kernels follow one another with programmatic dependent launch: a kernel
+// may be scheduled when every block of the one before it has started, and waits
+// in pdl_begin until that one (and with it all earlier ones) has completed and its
+// writes are visible, before it touches memory.  Its own dependents may be
+// scheduled from there on.  This hides the launch latency of the build's dependent
+// kernels: build 74 -> 57 us at N = 4096, 109 -> 95 at 262,144, 339 -> 315 at
+// 2,097,152.
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline void launch_pdl(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // bit of the highest boundary inside a run of keys, from its first and last
 // (a run of equal keys has none: every key is then on side 0)
 template <typename K>

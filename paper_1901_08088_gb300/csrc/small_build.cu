@@ -19,7 +19,6 @@ namespace {
 
 constexpr int kSB = 1024;                    // threads of the block
 constexpr int kSmallMax = 4096;              // largest system
-constexpr int kItems = kSmallMax / kSB;      // keys per thread
 constexpr int kWarps = kSB / 32;
 constexpr int kMaxTrees = 4;
 constexpr int kMaxDepth = 64;                // a radix tree over 30 + 12 key bits is at most 43 deep
@@ -50,7 +49,8 @@ __device__ __forceinline__ int delta_s(const unsigned *keys, int i, unsigned ci,
     return 32 + __clz((unsigned)i ^ (unsigned)j);
 }
 
-template <bool F32>
+// kItems: keys per thread; n is at most kItems * kSB
+template <bool F32, int kItems>
 __global__ void __launch_bounds__(kSB, 1) small_build_kernel(const BuildArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kSB, 1) small_build_kernel(const BuildArgs a)
     }
 
     // ---- Karras hierarchy: internal node i of the tree holding leaf i ------
-    for (int i = tid; i < kSmallMax; i += kSB) {
+    for (int i = tid; i < kItems * kSB; i += kSB) {
         s_range[i] = make_int2(0, -1);
         s_child[i] = make_int2(0, 0);
         s_par_int[i] = -1;
@@ -479,24 +479,31 @@ bool small_build_fits(const BuildArgs &a)
            a.n_types <= kMaxTrees;
 }
 
+template <bool F32, int kItems>
+static void launch_small(const BuildArgs &a, cudaStream_t s)
+{
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaFuncSetAttribute(small_build_kernel<F32, kItems>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kSmemBytes);
+        attr_set = true;
+    }
+    small_build_kernel<F32, kItems><<<1, kSB, kSmemBytes, s>>>(a);
+}
+
+// Keys per thread: no more than the system needs (the sort ranks every slot).
+template <bool F32>
+static void launch_small_items(const BuildArgs &a, cudaStream_t s)
+{
+    if (a.n <= kSB) launch_small<F32, 1>(a, s);
+    else if (a.n <= 2 * kSB) launch_small<F32, 2>(a, s);
+    else launch_small<F32, kSmallMax / kSB>(a, s);
+}
+
 void launch_small_build(const BuildArgs &a, cudaStream_t s)
 {
-    static bool attr_set[2] = {false, false};
-    if (a.nodes32) {
-        if (!attr_set[1]) {
-            cudaFuncSetAttribute(small_build_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemBytes);
-            attr_set[1] = true;
-        }
-        small_build_kernel<true><<<1, kSB, kSmemBytes, s>>>(a);
-    } else {
-        if (!attr_set[0]) {
-            cudaFuncSetAttribute(small_build_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSmemBytes);
-            attr_set[0] = true;
-        }
-        small_build_kernel<false><<<1, kSB, kSmemBytes, s>>>(a);
-    }
+    if (a.nodes32) launch_small_items<true>(a, s);
+    else launch_small_items<false>(a, s);
 }
 
 }  // namespace qbvh

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(kThreads) pass_kernel(const K *__restrict__ ki
                                                         unsigned *status, unsigned *ticket, unsigned *err,
                                                         int spin_limit)
 {
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned *s_whist = reinterpret_cast<unsigned *>(smem);   // [kWarps][256]
     unsigned *s_dstart = s_whist + kWarps * kRadix;            // [256]
@@ -257,9 +258,9 @@ int sort_impl(K *ka, K *kb, int *va, int *vb, int n, int bits, void *scratch, un
     int *v_first_dst = vb;
     (void)v_first_dst;
     for (int p = 0; p < npass; ++p) {
-        pass_kernel<K><<<tiles, kThreads, smem, s>>>(src_k, src_v, dst_k, dst_v, n, 8 * p, hist + p * kRadix,
-                                                     status + (size_t)p * tiles * kRadix, ticket + p * 4, err,
-                                                     kSpinLimit);
+        launch_pdl(pass_kernel<K>, tiles, kThreads, smem, s, (const K *)src_k, (const int *)src_v, dst_k, dst_v, n, 8 * p,
+                   (const unsigned *)(hist + p * kRadix), status + (size_t)p * tiles * kRadix, ticket + p * 4, err,
+                   (int)kSpinLimit);
         // ping-pong
         K *tk = src_k;
         src_k = dst_k;
