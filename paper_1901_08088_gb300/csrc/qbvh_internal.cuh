@@ -444,7 +444,6 @@ struct SortScratch {
     unsigned *counters;    // [passes] tile tickets
 };
 
-size_t sort_tile_items();
 int sort_num_tiles(int n);
 size_t sort_scratch_bytes(int n, int passes);
 // Sorts (key, value) pairs stably by the low `bits` bits of the key.  keys_a

@@ -23,14 +23,15 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-// keys per thread: 8 keeps 2048-key tiles, 27 KB of shared memory per block
-// and twice the blocks of 16 items (the pass is latency-bound: more resident
-// tiles hide more of the ranking and look-back latency)
-#ifndef QBVH_SORT_ITEMS
-#define QBVH_SORT_ITEMS 8
-#endif
-constexpr int kItems = QBVH_SORT_ITEMS;
-constexpr int kTile = kThreads * kItems;
+// Keys per thread.  8 keeps 2048-key tiles, 27 KB of shared memory per block and
+// twice the blocks of 16 items (the pass is latency-bound: more resident tiles
+// hide more of the ranking and look-back latency; N = 2,097,152, build with 16 / 8 /
+// 4 items: 364 / 317 / 326 us).  Below 200,000 keys a tile of 8 items leaves SMs
+// without one and its rows are ranked one after another: 4 items, build 104 -> 94
+// us at N = 131,072 and 56 -> 52 us at 4096 (98 against 94 us at 262,144).
+constexpr int kManyItems = 8;
+constexpr int kFewItems = 4;
+__host__ __device__ constexpr int items_for(int n) { return n < 200000 ? kFewItems : kManyItems; }
 constexpr int kRadix = 256;
 constexpr unsigned kFlagAgg = 1u << 30;
 constexpr unsigned kFlagPre = 2u << 30;
@@ -96,7 +97,7 @@ __device__ __forceinline__ unsigned block_excl_scan256(unsigned v, unsigned *s_w
     return before + x - v;
 }
 
-template <typename K>
+template <typename K, int kItems>
 __global__ void __launch_bounds__(kThreads) pass_kernel(const K *__restrict__ kin, const int *__restrict__ vin,
                                                         K *__restrict__ kout, int *__restrict__ vout, int n,
                                                         int shift, const unsigned *__restrict__ bucket_base,
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kThreads) pass_kernel(const K *__restrict__ ki
                                                         int spin_limit)
 {
     pdl_begin();
+    constexpr int kTile = kThreads * kItems;
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned *s_whist = reinterpret_cast<unsigned *>(smem);   // [kWarps][256]
     unsigned *s_dstart = s_whist + kWarps * kRadix;            // [256]
@@ -225,13 +227,13 @@ __global__ void __launch_bounds__(kThreads) pass_kernel(const K *__restrict__ ki
     }
 }
 
-template <typename K>
+template <typename K, int kItems>
 size_t pass_smem()
 {
-    return sizeof(unsigned) * (kWarps * kRadix + 2 * kRadix + 16) + (sizeof(K) + sizeof(int)) * kTile;
+    return sizeof(unsigned) * (kWarps * kRadix + 2 * kRadix + 16) + (sizeof(K) + sizeof(int)) * kThreads * kItems;
 }
 
-template <typename K>
+template <typename K, int kItems>
 int sort_impl(K *ka, K *kb, int *va, int *vb, int n, int bits, void *scratch, unsigned *err, bool prepared,
               cudaStream_t s)
 {
@@ -248,9 +250,9 @@ int sort_impl(K *ka, K *kb, int *va, int *vb, int n, int bits, void *scratch, un
         hist_kernel<K><<<hb, kThreads, 0, s>>>(ka, n, npass, hist);
     }
     static bool attr_set = false;
-    const size_t smem = pass_smem<K>();
+    const size_t smem = pass_smem<K, kItems>();
     if (!attr_set) {
-        cudaFuncSetAttribute(pass_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(pass_kernel<K, kItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         attr_set = true;
     }
     K *src_k = ka, *dst_k = kb;
@@ -258,7 +260,7 @@ int sort_impl(K *ka, K *kb, int *va, int *vb, int n, int bits, void *scratch, un
     int *v_first_dst = vb;
     (void)v_first_dst;
     for (int p = 0; p < npass; ++p) {
-        launch_pdl(pass_kernel<K>, tiles, kThreads, smem, s, (const K *)src_k, (const int *)src_v, dst_k, dst_v, n, 8 * p,
+        launch_pdl(pass_kernel<K, kItems>, tiles, kThreads, smem, s, (const K *)src_k, (const int *)src_v, dst_k, dst_v, n, 8 * p,
                    (const unsigned *)(hist + p * kRadix), status + (size_t)p * tiles * kRadix, ticket + p * 4, err,
                    (int)kSpinLimit);
         // ping-pong
@@ -274,9 +276,11 @@ int sort_impl(K *ka, K *kb, int *va, int *vb, int n, int bits, void *scratch, un
 
 }  // namespace
 
-size_t sort_tile_items() { return kTile; }
-
-int sort_num_tiles(int n) { return n <= 0 ? 1 : (n + kTile - 1) / kTile; }
+int sort_num_tiles(int n)
+{
+    const int tile = kThreads * items_for(n);
+    return n <= 0 ? 1 : (n + tile - 1) / tile;
+}
 
 size_t sort_scratch_bytes(int n, int passes)
 {
@@ -289,7 +293,7 @@ size_t sort_scratch_bytes(int n, int passes)
 // Every access stays inside the 2-tile buffers.  Returns the device error word.
 int sort_wait_selftest(int spin_limit, unsigned *err_out, cudaStream_t s)
 {
-    const int n = 2 * kTile;
+    const int n = 2 * kThreads * kManyItems;
     unsigned *kin = nullptr, *kout = nullptr, *misc = nullptr;
     int *vout = nullptr;
     const size_t misc_words = kRadix + 4 + 2 * kRadix + 1;   // bucket base, ticket, status of 2 tiles, err
@@ -307,9 +311,9 @@ int sort_wait_selftest(int spin_limit, unsigned *err_out, cudaStream_t s)
     cudaMemsetAsync(misc, 0, misc_words * sizeof(unsigned), s);
     const unsigned one = 1u;
     cudaMemcpyAsync(ticket, &one, sizeof one, cudaMemcpyHostToDevice, s);   // the block takes tile 1
-    const size_t smem = pass_smem<unsigned>();
-    cudaFuncSetAttribute(pass_kernel<unsigned>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    pass_kernel<unsigned><<<1, kThreads, smem, s>>>(kin, nullptr, kout, vout, n, 0, base, status, ticket, err,
+    const size_t smem = pass_smem<unsigned, kManyItems>();
+    cudaFuncSetAttribute(pass_kernel<unsigned, kManyItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    pass_kernel<unsigned, kManyItems><<<1, kThreads, smem, s>>>(kin, nullptr, kout, vout, n, 0, base, status, ticket, err,
                                                     spin_limit);   // tile 1: never scans
     cudaMemcpyAsync(err_out, err, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
     const cudaError_t e = cudaStreamSynchronize(s);
@@ -324,12 +328,16 @@ int radix_sort_pairs(bool wide, void *keys_a, void *keys_b, int *vals_a, int *va
                      void *scratch, unsigned *err, cudaStream_t s, bool prepared)
 {
     if (n <= 0) return 0;
-    if (wide)
-        return sort_impl<unsigned long long>(reinterpret_cast<unsigned long long *>(keys_a),
-                                             reinterpret_cast<unsigned long long *>(keys_b), vals_a, vals_b, n,
-                                             bits, scratch, err, prepared, s);
-    return sort_impl<unsigned>(reinterpret_cast<unsigned *>(keys_a), reinterpret_cast<unsigned *>(keys_b), vals_a,
-                               vals_b, n, bits, scratch, err, prepared, s);
+    using u64 = unsigned long long;
+    const bool few = items_for(n) == kFewItems;
+    if (wide) {
+        const auto sort = few ? sort_impl<u64, kFewItems> : sort_impl<u64, kManyItems>;
+        return sort(reinterpret_cast<u64 *>(keys_a), reinterpret_cast<u64 *>(keys_b), vals_a, vals_b, n, bits, scratch,
+                    err, prepared, s);
+    }
+    const auto sort = few ? sort_impl<unsigned, kFewItems> : sort_impl<unsigned, kManyItems>;
+    return sort(reinterpret_cast<unsigned *>(keys_a), reinterpret_cast<unsigned *>(keys_b), vals_a, vals_b, n, bits,
+                scratch, err, prepared, s);
 }
 
 }  // namespace qbvh
