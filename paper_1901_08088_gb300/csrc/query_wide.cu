@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(256, W == 1 && !(ONE && F64) ? 3 : 4) wide_que
     c.xi = me.x;
     c.yi = me.y;
     c.zi = me.z;
-    c.self = s;
+    c.self = active ? s : 0;   // an idle lane's tests read a valid particle too
     OutRow out{a.rows + (size_t)i * a.cap, a.cap, 0, 0};
     Walk w{0, 0, 0, -1};
     extern __shared__ __align__(16) unsigned char smem[];

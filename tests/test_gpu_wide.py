@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_1901_08088_gb300 import _lib
 from paper_1901_08088_gb300.qbvh import NeighborList
 
@@ -52,7 +53,7 @@ def _fluid(n, rho, seed):
     return x, float(L)
 
 
-@pytest.mark.parametrize("n", [64, 65, 1023, 1024, 1025, 7999, 8000, 8007, 32767, 32769, 59999, 60000, 60031, 70001])
+@pytest.mark.parametrize("n", [64, 65, 1023, 1024, 1025, 7999, 8000, 8007, 32767, 32769, 59999, 60000, 60031, 70001, 199999, 200001])
 def test_sizes(n):
     x, L = _fluid(n, 0.6, n)
     _same(_pos4(x), [0, n], [L], min(2.2, 0.45 * L))
@@ -103,3 +104,28 @@ def test_one_cluster(n):
     x = np.mod(rng.normal(0, 1.2 if n < 10000 else 6.0, (n, 3)), 60.0).astype(np.float32)
     x[x >= 60.0] = 0
     _same(_pos4(x), [0, n], [60.0], 0.6, cap=2048)
+
+
+@pytest.mark.parametrize("n", [4099, 20003, 65003])
+def test_double_precision_last_packet(n):
+    """Double-precision data whose last packet has idle lanes, pairs at the radius
+    near the box corner where those lanes' zero positions lie."""
+    rng = np.random.default_rng(n)
+    L = float((n / 0.6) ** (1 / 3))
+    x = rng.uniform(0, L, (n, 3))
+    r = np.float32(1.75)
+    k = min(64, n)
+    d = rng.normal(size=(k, 3))
+    x[:k] = np.mod(float(r) * (1 + 1e-9 * rng.integers(-2, 3, (k, 1))) * d / np.linalg.norm(d, axis=1, keepdims=True), L)
+    x[k] = 0.0
+    x[x >= L] = 0.0
+    pos = torch.from_numpy(np.concatenate([x, np.zeros((n, 1))], 1)).cuda()
+    nl = NeighborList()
+    nl.build_f64(pos, L, 1).query(float(r), cap=128)
+    rows, counts = (v.cpu().numpy() for v in nl.neighbors())
+    nl.close()
+    ro, co = oracle.nlist64(x, L, r, cap=rows.shape[1])
+    assert np.array_equal(counts, co)
+    big = np.iinfo(np.int32).max
+    live = np.arange(rows.shape[1])[None, :] < counts[:, None]
+    assert np.array_equal(np.sort(np.where(live, rows, big), 1), np.sort(np.where(live, ro[:, :rows.shape[1]], big), 1))
