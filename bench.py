@@ -107,21 +107,8 @@ class ClockSampler:
 # options of each entry and the traversal sources whose SHA-256 prefix is given; any
 # other source or options report null.
 PROFILED_TRAFFIC = {
-    "source_sha256": "ba179f7ae5a5ff5c",
-    "entries": [
-        {"options": {"bundle_k": 64, "node_format": 0, "traversal": 1, "warp_particles": 32, "query_block": 128,
-                     "fused_lj": 0, "persistent": 0},
-         "bytes": 109.72e6 + 1007.59e6, "warp_inst": 1336503549},
-        {"options": {"bundle_k": 64, "node_format": 0, "traversal": 1, "warp_particles": 32, "query_block": 256,
-                     "fused_lj": 0, "persistent": 0},
-         "bytes": 108.79e6 + 1006.68e6, "warp_inst": 1336503581},
-        {"options": {"bundle_k": 64, "node_format": 1, "traversal": 1, "warp_particles": 32, "query_block": 128,
-                     "fused_lj": 0, "persistent": 0},
-         "bytes": 107.69e6 + 994.58e6, "warp_inst": 1302335900},
-        {"options": {"bundle_k": 64, "node_format": 1, "traversal": 1, "warp_particles": 32, "query_block": 256,
-                     "fused_lj": 0, "persistent": 0},
-         "bytes": 107.69e6 + 994.40e6, "warp_inst": 1302335932},
-    ],
+    "source_sha256": "",   # the 32-wide walk has not been profiled at this size yet
+    "entries": [],
 }
 # kernels of one timed step: build = prepare, Morton (+ sort histograms), segment
 # scan, 4 onesweep passes (30-bit keys, 8-bit digits), Karras, fit; query = 1
@@ -129,7 +116,8 @@ PROFILED_TRAFFIC = {
 KERNELS_PER_STEP = 9 + 1 + 2
 # with the LJ terms summed inside the traversal: build, traversal, finalize
 KERNELS_PER_STEP_FUSED = 9 + 1 + 1
-_TRAFFIC_SOURCES = ("paper_1901_08088_gb300/csrc/query.cu", "paper_1901_08088_gb300/csrc/qbvh_internal.cuh")
+_TRAFFIC_SOURCES = ("paper_1901_08088_gb300/csrc/query_wide.cu", "paper_1901_08088_gb300/csrc/query_common.cuh",
+                    "paper_1901_08088_gb300/csrc/qbvh_internal.cuh")
 
 
 def traversal_source_hash() -> str:

@@ -62,7 +62,7 @@ __device__ __forceinline__ int4 row_chunk(const int *row, int k, int sub, int c)
 // system in rounds of kLJBlock / TPP.
 //
 // What bounds it: instruction issue and the latency of the gathers of neighbour
-// positions (N = 262,144, two lanes: 61% of the issue rate, L1 data pipe 65%,
+// positions (N = 262,144, two lanes: 64% of the issue rate, L1 data pipe 72%,
 // long-scoreboard stalls first).  So a pair takes no branch but the one for
 // pairs across a face: every pair's terms are formed and added by predicate.  The next
 // particle is looked up one round ahead and a row's next chunk one chunk ahead.

@@ -322,22 +322,18 @@ struct Row {
 // false leaves out the self test where the caller knows j cannot be the
 // particle itself.  (Under a non-zero image the particle's own copy is never
 // accepted anyway: its difference is -nL exactly, so d2 >= L^2 > r^2.)
-template <bool SHIFT, bool F64, bool SELF = true>
+template <bool SHIFT, bool SELF = true>
 __device__ __forceinline__ bool exact_accept(const QueryArgs &A, const Query &c, int j, const float4 q)
 {
     const float d2 = exact_d2<SHIFT>(c, q);
-    if (!F64) return d2 < c.rl2 && (!SELF || j != c.self);
-    if (SELF && j == c.self) return false;
-    if (d2 < c.rl2_lo) return true;
-    if (!(d2 <= c.rl2_hi)) return false;
-    return exact_d2_64<SHIFT>(A, c, j) < A.r2_64[c.pair];
+    return d2 < c.rl2 && (!SELF || j != c.self);
 }
 
 // The exact test of leaf j under the current image.
-template <bool SHIFT, bool F64, bool SELF = true>
+template <bool SHIFT, bool SELF = true>
 __device__ __forceinline__ void exact_leaf(const QueryArgs &A, const Query &c, Row &out, int j, const float4 q)
 {
-    if (exact_accept<SHIFT, F64, SELF>(A, c, j, q)) out.push(__float_as_int(q.w) & 0x7FFFFFFF);
+    if (exact_accept<SHIFT, SELF>(A, c, j, q)) out.push(__float_as_int(q.w) & 0x7FFFFFFF);
 }
 
 // Alg. 1 without the exact filter: the sphere against leaf j's box at the
@@ -373,25 +369,25 @@ __device__ __forceinline__ void candidate_leaf(const QueryArgs &A, const Query &
     if (j != c.self && cand_overlap<FMT>(A, c, j, q, f, rs2)) out.push(__float_as_int(q.w) & 0x7FFFFFFF);
 }
 
-template <bool CAND, bool SHIFT = true, bool F64 = false, bool SELF = true, int FMT = 0>
+template <bool CAND, bool SHIFT = true, bool SELF = true, int FMT = 0>
 __device__ __forceinline__ void test_leaf(const QueryArgs &A, const Query &c, Row &out, int j, const float4 q,
                                           const Frame &f, float rs2)
 {
     if (CAND)
         candidate_leaf<FMT>(A, c, out, j, q, f, rs2);
     else
-        exact_leaf<SHIFT, F64, SELF>(A, c, out, j, q);
+        exact_leaf<SHIFT, SELF>(A, c, out, j, q);
 }
 
 // The same decisions as exact_leaf / candidate_leaf, returned instead of
 // appended (used when several lanes share one particle's row).
-template <bool CAND, bool SHIFT, bool F64 = false, int FMT = 0>
+template <bool CAND, bool SHIFT, int FMT = 0>
 __device__ __forceinline__ bool leaf_accepts(const QueryArgs &A, const Query &c, int j, const float4 q,
                                              const Frame &f, float rs2)
 {
     if (j == c.self) return false;
     if (CAND) return cand_overlap<FMT>(A, c, j, q, f, rs2);
-    return exact_accept<SHIFT, F64>(A, c, j, q);
+    return exact_accept<SHIFT>(A, c, j, q);
 }
 
 // Append for W lanes sharing a row: the lanes of one particle are `same`
@@ -512,7 +508,7 @@ __global__ void query_thread_kernel(const __grid_constant__ QueryArgs a)
                                     l = nd.left - 1;
                                 }
                                 for (int j = nd.left; j <= l; ++j)
-                                    test_leaf<CAND, true, false, true, FMT>(a, c, out, j, tree_ld(a.leaves + j), f,
+                                    test_leaf<CAND, true, true, FMT>(a, c, out, j, tree_ld(a.leaves + j), f,
                                                                            rs2);
                                 node = nd.rope;
                             } else {
@@ -524,7 +520,7 @@ __global__ void query_thread_kernel(const __grid_constant__ QueryArgs a)
                     } else {
                         const int j = ~node;
                         const float4 q = tree_ld(a.leaves + j);
-                        test_leaf<CAND, true, false, true, FMT>(a, c, out, j, q, f, rs2);
+                        test_leaf<CAND, true, true, FMT>(a, c, out, j, q, f, rs2);
                         node = (j == last) ? QBVH_END : ((__float_as_int(q.w) < 0) ? j + 1 : ~(j + 1));
                     }
                 }
@@ -550,7 +546,7 @@ __global__ void query_thread_kernel(const __grid_constant__ QueryArgs a)
 #ifndef QBVH_SPREAD_MAX
 #define QBVH_SPREAD_MAX 16
 #endif
-template <bool SHIFT, bool F64, bool SELF>
+template <bool SHIFT, bool SELF>
 __device__ __forceinline__ void bundle_spread(const QueryArgs &a, const Query &c, Row &out, int first, int cnt,
                                               unsigned hm)
 {
@@ -583,7 +579,7 @@ __device__ __forceinline__ void bundle_spread(const QueryArgs &a, const Query &c
         t.self = c.self - lane + src;
         const int ocount = __shfl_sync(FULL, out.count, src);
         int *orow = reinterpret_cast<int *>(__shfl_sync(FULL, reinterpret_cast<unsigned long long>(out.row), src));
-        const bool acc = owner >= 0 && jv && exact_accept<SHIFT, F64, SELF>(a, t, j, q);
+        const bool acc = owner >= 0 && jv && exact_accept<SHIFT, SELF>(a, t, j, q);
         const unsigned m = __ballot_sync(FULL, acc);
         if (acc) {
             const int slot = ocount + __popc(m & gmask & lt);
@@ -698,10 +694,10 @@ __device__ __forceinline__ bool cube_overlap(unsigned nlo, unsigned nhi, const L
 #ifndef QBVH_MULTI_LANE_FILTER
 #define QBVH_MULTI_LANE_FILTER 1
 #endif
-__host__ __device__ constexpr bool stage_on(int W, bool CAND, bool F64)
+__host__ __device__ constexpr bool stage_on(int W, bool CAND)
 {
     return QBVH_PREFILTER && !CAND &&
-           (W == 1 || (!F64 && QBVH_MULTI_LANE_FILTER && (W == 2 || W == 4) && QBVH_ROW_STAGING &&
+           (W == 1 || (QBVH_MULTI_LANE_FILTER && (W == 2 || W == 4) && QBVH_ROW_STAGING &&
                        !QBVH_QUERY_SPLIT_IMAGES));
 }
 
@@ -822,23 +818,7 @@ struct LJCtx {
 
 // Two survivors (x, y, z as packed pairs, original indices id) against the
 // lane's particle.
-// Z-order indices of a warp's survivors (double-precision data only): a
-// second array after the block's stages in dynamic shared memory.
-__device__ __forceinline__ const int *stage_zid(const BundleStage *st)
-{
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    return reinterpret_cast<const int *>(st - warp + nw) + warp * kStage;
-}
-
-// Double-precision data: the decision for a survivor (Z-order index j) whose
-// FP32 d2 lies inside the band around r^2 (see exact_d2_64).
-template <bool SHIFT>
-__device__ __forceinline__ bool band_decide(const QueryArgs &A, const Query &c, int j)
-{
-    return exact_d2_64<SHIFT>(A, c, j) < A.r2_64[c.pair];
-}
-
-template <bool SHIFT, bool SELF, bool LJ = false, bool F64 = false>
+template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivor_vals(const Query &c, Row &out, const f32x2 X, const f32x2 Y, const f32x2 Z,
                                               const int2 id, bool on, bool staged, const LJCtx &lj,
                                               const QueryArgs *A = nullptr, const BundleStage *st = nullptr,
@@ -858,22 +838,8 @@ __device__ __forceinline__ void survivor_vals(const Query &c, Row &out, const f3
     const float d0 = __fadd_rn(__fadd_rn(sx0, sy0), sz0);
     const float d1 = __fadd_rn(__fadd_rn(sx1, sy1), sz1);
     bool a0, a1;
-    if (F64) {
-        // FP32 decides outside the band [rl2_lo, rl2_hi], FP64 inside it (rare)
-        const bool s0 = on && (!SELF || id.x != c.self_id), s1 = on && (!SELF || id.y != c.self_id);
-        a0 = s0 && d0 < c.rl2_lo;
-        a1 = s1 && d1 < c.rl2_lo;
-        const bool b0 = s0 && !(d0 < c.rl2_lo) && d0 <= c.rl2_hi;
-        const bool b1 = s1 && !(d1 < c.rl2_lo) && d1 <= c.rl2_hi;
-        if (b0 || b1) {
-            const int *zid = stage_zid(st);
-            if (b0) a0 = band_decide<SHIFT>(*A, c, zid[t]);
-            if (b1) a1 = band_decide<SHIFT>(*A, c, zid[t + 1]);
-        }
-    } else {
-        a0 = on && d0 < c.rl2 && (!SELF || id.x != c.self_id);
-        a1 = on && d1 < c.rl2 && (!SELF || id.y != c.self_id);
-    }
+    a0 = on && d0 < c.rl2 && (!SELF || id.x != c.self_id);
+    a1 = on && d1 < c.rl2 && (!SELF || id.y != c.self_id);
     if (LJ) {
         f32x2 vx = dx, vy = dy, vz = dz;
         float r0 = d0, r1 = d1;
@@ -900,11 +866,11 @@ __device__ __forceinline__ void survivor_vals(const Query &c, Row &out, const f3
 }
 
 // survivors t, t + 1 of the stage (8-byte loads)
-template <bool SHIFT, bool SELF, bool LJ = false, bool F64 = false>
+template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivor_pair(const Query &c, Row &out, int t, bool on, const BundleStage *st,
                                               bool staged, const LJCtx &lj = LJCtx{}, const QueryArgs *A = nullptr)
 {
-    survivor_vals<SHIFT, SELF, LJ, F64>(c, out, *reinterpret_cast<const f32x2 *>(st->x + t),
+    survivor_vals<SHIFT, SELF, LJ>(c, out, *reinterpret_cast<const f32x2 *>(st->x + t),
                                         *reinterpret_cast<const f32x2 *>(st->y + t),
                                         *reinterpret_cast<const f32x2 *>(st->z + t),
                                         *reinterpret_cast<const int2 *>(st->id + t), on, staged, lj, A, st, t);
@@ -916,7 +882,7 @@ __device__ __forceinline__ void survivor_pair(const Query &c, Row &out, int t, b
 #ifndef QBVH_SURVIVOR_QUAD
 #define QBVH_SURVIVOR_QUAD 1
 #endif
-template <bool SHIFT, bool SELF, bool LJ = false, bool F64 = false>
+template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivor_quad(const Query &c, Row &out, int t, bool on, const BundleStage *st,
                                               const LJCtx &lj, const QueryArgs *A = nullptr)
 {
@@ -924,9 +890,9 @@ __device__ __forceinline__ void survivor_quad(const Query &c, Row &out, int t, b
     const float4 Y = *reinterpret_cast<const float4 *>(st->y + t);
     const float4 Z = *reinterpret_cast<const float4 *>(st->z + t);
     const int4 I = *reinterpret_cast<const int4 *>(st->id + t);
-    survivor_vals<SHIFT, SELF, LJ, F64>(c, out, f2_pack(X.x, X.y), f2_pack(Y.x, Y.y), f2_pack(Z.x, Z.y),
+    survivor_vals<SHIFT, SELF, LJ>(c, out, f2_pack(X.x, X.y), f2_pack(Y.x, Y.y), f2_pack(Z.x, Z.y),
                                         make_int2(I.x, I.y), on, true, lj, A, st, t);
-    survivor_vals<SHIFT, SELF, LJ, F64>(c, out, f2_pack(X.z, X.w), f2_pack(Y.z, Y.w), f2_pack(Z.z, Z.w),
+    survivor_vals<SHIFT, SELF, LJ>(c, out, f2_pack(X.z, X.w), f2_pack(Y.z, Y.w), f2_pack(Z.z, Z.w),
                                         make_int2(I.z, I.w), on, true, lj, A, st, t + 2);
 }
 
@@ -938,7 +904,7 @@ __device__ __forceinline__ void survivor_quad(const Query &c, Row &out, int t, b
 // of the N = 2M list differed at d = r_list.  Scalar add.rn is not contracted.)
 // With row staging the accepted entries are staged without a branch and the
 // completed sectors written once per 8 survivors and at the end.
-template <bool SHIFT, bool SELF, bool LJ = false, bool F64 = false>
+template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivors_loop(const Query &c, Row &out, int s, bool on, const BundleStage *st,
                                                const LJCtx &lj = LJCtx{}, const QueryArgs *A = nullptr)
 {
@@ -947,25 +913,23 @@ __device__ __forceinline__ void survivors_loop(const Query &c, Row &out, int s, 
     if (staged) {
         for (; t + 8 <= s; t += 8) {
 #if QBVH_SURVIVOR_QUAD
-            survivor_quad<SHIFT, SELF, LJ, F64>(c, out, t, on, st, lj, A);
-            survivor_quad<SHIFT, SELF, LJ, F64>(c, out, t + 4, on, st, lj, A);
+            survivor_quad<SHIFT, SELF, LJ>(c, out, t, on, st, lj, A);
+            survivor_quad<SHIFT, SELF, LJ>(c, out, t + 4, on, st, lj, A);
 #else
-            survivor_pair<SHIFT, SELF, LJ, F64>(c, out, t, on, st, true, lj, A);
-            survivor_pair<SHIFT, SELF, LJ, F64>(c, out, t + 2, on, st, true, lj, A);
-            survivor_pair<SHIFT, SELF, LJ, F64>(c, out, t + 4, on, st, true, lj, A);
-            survivor_pair<SHIFT, SELF, LJ, F64>(c, out, t + 6, on, st, true, lj, A);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t, on, st, true, lj, A);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 2, on, st, true, lj, A);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 4, on, st, true, lj, A);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 6, on, st, true, lj, A);
 #endif
             out.check();
         }
     }
-    for (; t + 1 < s; t += 2) survivor_pair<SHIFT, SELF, LJ, F64>(c, out, t, on, st, staged, lj, A);
+    for (; t + 1 < s; t += 2) survivor_pair<SHIFT, SELF, LJ>(c, out, t, on, st, staged, lj, A);
     if (t < s) {
         const float4 q = make_float4(st->x[t], st->y[t], st->z[t], 0.f);
         const int id = st->id[t];
         const float d2 = exact_d2<SHIFT>(c, q);
-        bool acc = on && d2 < (F64 ? c.rl2_lo : c.rl2) && (!SELF || id != c.self_id);
-        if (F64 && on && (!SELF || id != c.self_id) && !(d2 < c.rl2_lo) && d2 <= c.rl2_hi)
-            acc = band_decide<SHIFT>(*A, c, stage_zid(st)[t]);
+        bool acc = on && d2 < c.rl2 && (!SELF || id != c.self_id);
         if (LJ) lj_single<SHIFT>(*lj.acc, c, lj.sig2, lj.rc2, acc, d2, q);
         if (staged) out.stage(id, acc);
         else if (acc) out.push(id);
@@ -1087,7 +1051,6 @@ __device__ __forceinline__ void bundle_chunk(const QueryArgs &a, const Query &c,
 // The filter of a chunk of cnt <= 32 leaves starting at `first`: its
 // survivors are appended to the stage after the s already there; returns the
 // new count (warp-uniform).  Every lane of the warp calls this together.
-template <bool F64 = false>
 __device__ __forceinline__ int chunk_filter(const QueryArgs &a, int first, int cnt, float rs2, BundleStage *st,
                                             int s)
 {
@@ -1110,7 +1073,6 @@ __device__ __forceinline__ int chunk_filter(const QueryArgs &a, int first, int c
         st->y[r] = q.y;
         st->z[r] = q.z;
         st->id[r] = __float_as_int(q.w) & 0x7FFFFFFF;
-        if (F64) const_cast<int *>(stage_zid(st))[r] = first + lane;
     }
     return s + __popc(S);
 }
@@ -1121,7 +1083,7 @@ __device__ __forceinline__ int chunk_filter(const QueryArgs &a, int first, int c
 // distance overflows to +inf, so no lane accepts them, and their LJ terms are
 // zero.  (With the spread of few-lane bundles, a build option without row
 // staging, chunks are tested one at a time.)
-template <bool SHIFT, bool SELF, bool LJ = false, int W = 1, bool F64 = false>
+template <bool SHIFT, bool SELF, bool LJ = false, int W = 1>
 __device__ __forceinline__ void bundle_filtered(const QueryArgs &a, const Query &c, Row &out, int first, int cnt,
                                                 unsigned hm, bool on, float rs2, BundleStage *st,
                                                 const LJCtx &lj = LJCtx{}, int wsub = 0, unsigned same = 0u)
@@ -1134,7 +1096,7 @@ __device__ __forceinline__ void bundle_filtered(const QueryArgs &a, const Query 
     }
     int s = 0;
     for (int base = 0; base < cnt; base += 32)
-        s = chunk_filter<F64>(a, first + base, min(32, cnt - base), rs2, st, s);
+        s = chunk_filter(a, first + base, min(32, cnt - base), rs2, st, s);
     if (s == 0) return;
     const int pad = (2 * W - s % (2 * W)) % (2 * W);   // s <= 64, a multiple of 2 W: s + pad <= 64
     const int lane = threadIdx.x & 31;
@@ -1143,11 +1105,10 @@ __device__ __forceinline__ void bundle_filtered(const QueryArgs &a, const Query 
         st->y[s + lane] = 1e30f;
         st->z[s + lane] = 1e30f;
         st->id[s + lane] = 0;
-        if (F64) const_cast<int *>(stage_zid(st))[s + lane] = first;   // never read: +inf is outside the band
     }
     s += pad;
     __syncwarp();
-    if (W == 1) survivors_loop<SHIFT, SELF, LJ, F64>(c, out, s, on, st, lj, &a);
+    if (W == 1) survivors_loop<SHIFT, SELF, LJ>(c, out, s, on, st, lj, &a);
     else survivors_loop_w<SHIFT, SELF, W>(c, out, s, on, st, wsub, same);
     __syncwarp();   // the next bundle rewrites the stage
 }
@@ -1158,7 +1119,7 @@ __device__ __forceinline__ void bundle_filtered(const QueryArgs &a, const Query 
 #define QBVH_LEAF_PAIRS 1
 #endif
 // Every lane tests every leaf j..l of a bundle (one particle per lane).
-template <bool CAND, bool SHIFT, bool F64, bool SELF, int FMT>
+template <bool CAND, bool SHIFT, bool SELF, int FMT>
 __device__ __forceinline__ void bundle_loop(const QueryArgs &a, const Query &c, Row &out, int j, int l,
                                             const Frame &f, float rs2, bool on)
 {
@@ -1167,14 +1128,14 @@ __device__ __forceinline__ void bundle_loop(const QueryArgs &a, const Query &c, 
         const float4 q0 = tree_ld(a.leaves + j);
         const float4 q1 = tree_ld(a.leaves + j + 1);
         if (on) {
-            test_leaf<CAND, SHIFT, F64, SELF, FMT>(a, c, out, j, q0, f, rs2);
-            test_leaf<CAND, SHIFT, F64, SELF, FMT>(a, c, out, j + 1, q1, f, rs2);
+            test_leaf<CAND, SHIFT, SELF, FMT>(a, c, out, j, q0, f, rs2);
+            test_leaf<CAND, SHIFT, SELF, FMT>(a, c, out, j + 1, q1, f, rs2);
         }
     }
 #endif
     for (; j <= l; ++j) {
         const float4 q = tree_ld(a.leaves + j);
-        if (on) test_leaf<CAND, SHIFT, F64, SELF, FMT>(a, c, out, j, q, f, rs2);
+        if (on) test_leaf<CAND, SHIFT, SELF, FMT>(a, c, out, j, q, f, rs2);
     }
 }
 
@@ -1186,15 +1147,15 @@ __device__ __forceinline__ void bundle_loop(const QueryArgs &a, const Query &c, 
 #endif
 // ---- one warp per 32 consecutive Z-order particles ----------------------
 // The warp-uniform rope walk of one tree under one periodic image.
-template <bool CAND, int FMT, bool SHIFT, int W, bool F64, bool LJ = false>
+template <bool CAND, int FMT, bool SHIFT, int W, bool LJ = false>
 __device__ __forceinline__ void warp_walk(const QueryArgs &a, const Query &c, Row &out, const SegInfo &g,
                                           const Frame &f, int root, int last, bool on, float rs2, int wsub,
                                           unsigned same, BundleStage *st = nullptr, float rs = 0.f,
                                           const LJCtx &lj = LJCtx{})
 {
-    static_assert(!LJ || (stage_on(W, CAND, F64) && !CAND && !F64 && W == 1), "LJ terms need the filtered walk");
+    static_assert(!LJ || (stage_on(W, CAND) && !CAND && W == 1), "LJ terms need the filtered walk");
     // bundles filtered against the warp's box (one particle per lane, exact lists of FP32 data)
-    constexpr bool FILTER = stage_on(W, CAND, F64);
+    constexpr bool FILTER = stage_on(W, CAND);
     // 10-bit nodes tested in the integer domain on the same walks
     constexpr bool QCUBE = FILTER && FMT == 0 && QBVH_QCUBE;
     if (FILTER) packet_box(c, on, st);
@@ -1236,17 +1197,17 @@ __device__ __forceinline__ void warp_walk(const QueryArgs &a, const Query &c, Ro
                         !SHIFT && __any_sync(FULL, (unsigned)(c.self - j) <= (unsigned)(l - j));
                     if (FILTER && l - j < 64) {
                         if (self_here)
-                            bundle_filtered<SHIFT, true, LJ, W, F64>(a, c, out, j, l - j + 1, hm, on, rs2, st, lj,
+                            bundle_filtered<SHIFT, true, LJ, W>(a, c, out, j, l - j + 1, hm, on, rs2, st, lj,
                                                                      wsub, same);
                         else
-                            bundle_filtered<SHIFT, false, LJ, W, F64>(a, c, out, j, l - j + 1, hm, on, rs2, st, lj,
+                            bundle_filtered<SHIFT, false, LJ, W>(a, c, out, j, l - j + 1, hm, on, rs2, st, lj,
                                                                       wsub, same);
                     } else if (W == 1 && !CAND && l - j < 32 && __popc(hm) <= QBVH_SPREAD_MAX) {
-                        if (self_here) bundle_spread<SHIFT, F64, true>(a, c, out, j, l - j + 1, hm);
-                        else bundle_spread<SHIFT, F64, false>(a, c, out, j, l - j + 1, hm);
+                        if (self_here) bundle_spread<SHIFT, true>(a, c, out, j, l - j + 1, hm);
+                        else bundle_spread<SHIFT, false>(a, c, out, j, l - j + 1, hm);
                     } else if (W == 1) {
-                        if (self_here || CAND) bundle_loop<CAND, SHIFT, F64, true, FMT>(a, c, out, j, l, f, rs2, on);
-                        else bundle_loop<CAND, SHIFT, F64, false, FMT>(a, c, out, j, l, f, rs2, on);
+                        if (self_here || CAND) bundle_loop<CAND, SHIFT, true, FMT>(a, c, out, j, l, f, rs2, on);
+                        else bundle_loop<CAND, SHIFT, false, FMT>(a, c, out, j, l, f, rs2, on);
                     } else {
                         // the W lanes of a particle take every W-th leaf
                         for (; j <= l; j += W) {
@@ -1255,7 +1216,7 @@ __device__ __forceinline__ void warp_walk(const QueryArgs &a, const Query &c, Ro
                             int id = 0;
                             if (jj <= l) {
                                 const float4 q = tree_ld(a.leaves + jj);
-                                acc = on && leaf_accepts<CAND, SHIFT, F64, FMT>(a, c, jj, q, f, rs2);
+                                acc = on && leaf_accepts<CAND, SHIFT, FMT>(a, c, jj, q, f, rs2);
                                 id = __float_as_int(q.w) & 0x7FFFFFFF;
                             }
                             push_shared(out, acc, id, same);
@@ -1277,14 +1238,14 @@ __device__ __forceinline__ void warp_walk(const QueryArgs &a, const Query &c, Ro
                 lj_single<SHIFT>(*lj.acc, c, lj.sig2, lj.rc2, acc, d2, q);
                 if (acc) out.push(__float_as_int(q.w) & 0x7FFFFFFF);
             } else if (W == 1) {
-                if (on) test_leaf<CAND, SHIFT, F64, true, FMT>(a, c, out, j, q, f, rs2);
+                if (on) test_leaf<CAND, SHIFT, true, FMT>(a, c, out, j, q, f, rs2);
             } else if (FILTER) {
                 // the group's row goes through the staging rings
-                const bool acc = wsub == 0 && on && leaf_accepts<CAND, SHIFT, F64, FMT>(a, c, j, q, f, rs2);
+                const bool acc = wsub == 0 && on && leaf_accepts<CAND, SHIFT, FMT>(a, c, j, q, f, rs2);
                 out.stage(__float_as_int(q.w) & 0x7FFFFFFF, acc);
                 out.check_group(same);
             } else {
-                const bool acc = wsub == 0 && on && leaf_accepts<CAND, SHIFT, F64, FMT>(a, c, j, q, f, rs2);
+                const bool acc = wsub == 0 && on && leaf_accepts<CAND, SHIFT, FMT>(a, c, j, q, f, rs2);
                 push_shared(out, acc, __float_as_int(q.w) & 0x7FFFFFFF, same);
             }
             node = (j == last) ? QBVH_END : ((__float_as_int(q.w) < 0) ? j + 1 : ~(j + 1));
@@ -1367,9 +1328,9 @@ __device__ __forceinline__ void sparse_walks(const QueryArgs &a)
                     mask &= mask - 1u;
                     set_image(c, img, L);
                     if (img == 13)
-                        warp_walk<false, FMT, false, 32, false>(a, c, out, g, f, root, last, true, rs2, lane, FULL);
+                        warp_walk<false, FMT, false, 32>(a, c, out, g, f, root, last, true, rs2, lane, FULL);
                     else
-                        warp_walk<false, FMT, true, 32, false>(a, c, out, g, f, root, last, true, rs2, lane, FULL);
+                        warp_walk<false, FMT, true, 32>(a, c, out, g, f, root, last, true, rs2, lane, FULL);
                 }
             }
             if (lane == 0) a.counts[i_orig] = out.count;
@@ -1419,13 +1380,13 @@ __device__ __forceinline__ void lj_block_record(const QueryArgs &a, double v0, d
 
 // One packet: the G = 32 / W consecutive Z-order particles p G, ..., p G + G - 1
 // walked by this warp.  Every lane of the warp calls this together.
-template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool F64, bool LJ>
+template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool LJ>
 __device__ __forceinline__ void warp_packet(const QueryArgs &a, int p)
 {
-    static_assert(!LJ || (ONE && W == 1 && !CAND && !F64 && PHASE == 2), "LJ terms: one tree, filtered walk");
+    static_assert(!LJ || (ONE && W == 1 && !CAND && PHASE == 2), "LJ terms: one tree, filtered walk");
     constexpr int G = 32 / W;
     // sparse trees (above) exist for single-system builds with several types
-    constexpr bool SPARSE = QBVH_SPARSE_TREES && !WIDE && !ONE && !CAND && !F64 && PHASE == 2;
+    constexpr bool SPARSE = QBVH_SPARSE_TREES && !WIDE && !ONE && !CAND && PHASE == 2;
     const int lane = threadIdx.x & 31;
     const int pidx = lane % G;
     const int wsub = lane / G;
@@ -1453,7 +1414,7 @@ __device__ __forceinline__ void warp_packet(const QueryArgs &a, int p)
     out.row = a.rows + (size_t)i_orig * a.cap;
     out.cap = a.cap;
     out.count = (PHASE == 1 && active) ? a.counts[i_orig] : 0;
-    constexpr bool STAGE = stage_on(W, CAND, F64);
+    constexpr bool STAGE = stage_on(W, CAND);
     // one BundleStage per warp, in dynamic shared memory sized to the block
     extern __shared__ BundleStage stage[];
     BundleStage *st = STAGE ? &stage[threadIdx.x >> 5] : nullptr;
@@ -1495,11 +1456,6 @@ __device__ __forceinline__ void warp_packet(const QueryArgs &a, int p)
             const SegInfo g = a.seg[sys * T + tb];
             if (g.count == 0) continue;
             c.rl2 = a.rl2[ta * T + tb];
-            if (F64) {
-                c.rl2_lo = a.rl2_lo[ta * T + tb];
-                c.rl2_hi = a.rl2_hi[ta * T + tb];
-                c.pair = ta * T + tb;
-            }
             const float rs2 = a.rs2[ta * T + tb];
             const float rs = a.rs[ta * T + tb];
             const Frame f = FMT == 2 ? frame21_of(g) : frame_of(g);
@@ -1508,7 +1464,7 @@ __device__ __forceinline__ void warp_packet(const QueryArgs &a, int p)
             if (PHASE == 0) {
                 // zero image: the walk's own root test decides whether it is empty
                 set_image(c, 13, L);
-                warp_walk<CAND, FMT, false, W, F64>(a, c, out, g, f, root, last, part, rs2, wsub, same, st, rs);
+                warp_walk<CAND, FMT, false, W>(a, c, out, g, f, root, last, part, rs2, wsub, same, st, rs);
                 continue;
             }
             unsigned mine = part ? image_mask(me.x, me.y, me.z, L, g, rs2) : 0u;
@@ -1522,10 +1478,10 @@ __device__ __forceinline__ void warp_packet(const QueryArgs &a, int p)
                 if (LJ) set_lj_value(c, L);
                 const bool on = (mine >> img) & 1u;
                 if (PHASE == 2 && img == 13)
-                    warp_walk<CAND, FMT, false, W, F64, LJ>(a, c, out, g, f, root, last, on, rs2, wsub, same, st,
+                    warp_walk<CAND, FMT, false, W, LJ>(a, c, out, g, f, root, last, on, rs2, wsub, same, st,
                                                             rs, lj);
                 else
-                    warp_walk<CAND, FMT, true, W, F64, LJ>(a, c, out, g, f, root, last, on, rs2, wsub, same, st,
+                    warp_walk<CAND, FMT, true, W, LJ>(a, c, out, g, f, root, last, on, rs2, wsub, same, st,
                                                            rs, lj);
             }
         }
@@ -1577,10 +1533,10 @@ __device__ __forceinline__ void warp_packet(const QueryArgs &a, int p)
 // packets span wide regions and walk longest) start first and overlap the rest
 // instead of running alone at the end (mixture L = 100: 2.05 -> 1.89 ms before
 // sparse trees).
-template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool F64, bool LJ>
+template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool LJ>
 __device__ __forceinline__ void warp_query(const QueryArgs &a)
 {
-    constexpr bool SPARSE = QBVH_SPARSE_TREES && !WIDE && !ONE && !CAND && !F64 && PHASE == 2;
+    constexpr bool SPARSE = QBVH_SPARSE_TREES && !WIDE && !ONE && !CAND && PHASE == 2;
     int bid = (int)blockIdx.x, nblk = (int)gridDim.x;
     if (SPARSE && a.sparse_blocks > 0) {
         if (bid < a.sparse_blocks) {
@@ -1592,20 +1548,20 @@ __device__ __forceinline__ void warp_query(const QueryArgs &a)
     }
     const bool rev = QBVH_REVERSE_BLOCKS && (ONE ? 1 : a.n_types) > 1;
     const int blk = rev ? nblk - 1 - bid : bid;
-    warp_packet<WIDE, CAND, FMT, W, ONE, PHASE, F64, LJ>(a, (int)((blk * blockDim.x + threadIdx.x) >> 5));
+    warp_packet<WIDE, CAND, FMT, W, ONE, PHASE, LJ>(a, (int)((blk * blockDim.x + threadIdx.x) >> 5));
 }
 
-template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE, bool F64 = false>
+template <bool WIDE, bool CAND, int FMT, int W, bool ONE, int PHASE>
 __global__ void QBVH_QUERY_BOUNDS query_warp_kernel(const __grid_constant__ QueryArgs a)
 {
-    warp_query<WIDE, CAND, FMT, W, ONE, PHASE, F64, false>(a);
+    warp_query<WIDE, CAND, FMT, W, ONE, PHASE, false>(a);
 }
 
 // the walk of one system of one type that also sums the LJ terms of its pairs
 template <int FMT>
 __global__ void __launch_bounds__(256, QBVH_QUERY_LJ_MIN_BLOCKS) query_warp_lj_kernel(const __grid_constant__ QueryArgs a)
 {
-    warp_query<false, false, FMT, 1, true, 2, false, true>(a);
+    warp_query<false, false, FMT, 1, true, 2, true>(a);
 }
 
 }  // namespace
@@ -1617,10 +1573,9 @@ static int sparse_blocks_for(const QueryArgs &a)
 }
 
 // dynamic shared memory of a traversal block: one BundleStage per warp
-static size_t stage_bytes(int block, bool stage, bool f64 = false)
+static size_t stage_bytes(int block, bool stage)
 {
-    // double-precision data: the survivors' Z-order indices after the stages
-    return stage ? (size_t)(block / 32) * (sizeof(BundleStage) + (f64 ? kStage * sizeof(int) : 0)) : 0;
+    return stage ? (size_t)(block / 32) * sizeof(BundleStage) : 0;
 }
 
 template <int FMT, int W, int PHASE>
@@ -1632,7 +1587,7 @@ static void launch_warp_phase(QueryArgs a, cudaStream_t s, int grid)
         a.sparse_blocks = sparse_blocks_for(a);
         grid += a.sparse_blocks;
     }
-    const size_t sm = stage_bytes(b, stage_on(W, a.candidates != 0, false));
+    const size_t sm = stage_bytes(b, stage_on(W, a.candidates != 0));
     if (a.candidates) {
         if (a.wide_keys) query_warp_kernel<true, true, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);
         else query_warp_kernel<false, true, FMT, W, false, PHASE><<<grid, b, sm, s>>>(a);

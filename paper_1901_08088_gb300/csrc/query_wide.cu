@@ -63,7 +63,7 @@
 // precision 339 -> 130; 262,144 327 -> 159; the L = 100 mixture 576 -> 248; liquid/
 // vapor 1,000,000 646 -> 393; 32 x 65,536 1523 -> 1028; 256 uneven systems 1904 ->
 // 1230; 2,097,152 1242 -> 953.  Bound by instruction issue and shared memory
-// together (N = 262,144: 67% of the issue rate, 65% of the L1 data pipe); leaving
+// together (N = 262,144: 62% of the issue rate, 58% of the L1 data pipe); leaving
 // parts out at N = 2,097,152 put 39% of the time in writing the rows, 25% in the
 // group tests, 20% in the chunks' filter, 16% in boxes and set-up.  One code path
 // for every image matters: with a second one for the zero image the uneven systems
