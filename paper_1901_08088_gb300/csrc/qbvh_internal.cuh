@@ -28,6 +28,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #define QBVH_END ((int)0x80000000)
 
 // device error word bits
@@ -410,6 +412,22 @@ inline void launch_pdl(void (*kernel)(P...), int grid, int block, size_t smem, c
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Permission for a kernel to take `bytes` of dynamic shared memory (more than 48 KB
+// need it), given once per device: it belongs to the kernel on the current device.
+// `bytes` is the most that any launch of the kernel takes, so that no thread takes
+// away what another one is about to use.  A refusal shows in the launch's status.
+template <auto Kernel>
+inline void allow_smem(size_t bytes)
+{
+    constexpr int kMaxDev = 64;
+    static std::atomic<bool> given[kMaxDev];
+    int dev = -1;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDev;
+    if (known && given[dev].load(std::memory_order_acquire)) return;
+    if (cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess && known)
+        given[dev].store(true, std::memory_order_release);
 }
 
 // bit of the highest boundary inside a run of keys, from its first and last

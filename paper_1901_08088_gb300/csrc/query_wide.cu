@@ -637,8 +637,7 @@ void launch_w(const QueryArgs &a, int extra, cudaStream_t s)
     const int grid = (packets + warps - 1) / warps + extra;
     const size_t smem = warps * stage_size<W>();
     // blocks of 224 and 256 threads exceed the 48 KB that need no opt-in
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(wide_query_kernel<ONE, F64, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 48 * 1024) allow_smem<wide_query_kernel<ONE, F64, W>>(8 * stage_size<W>());
     wide_query_kernel<ONE, F64, W><<<grid, a.block, smem, s>>>(a);
 }
 

@@ -482,12 +482,7 @@ bool small_build_fits(const BuildArgs &a)
 template <bool F32, int kItems>
 static void launch_small(const BuildArgs &a, cudaStream_t s)
 {
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(small_build_kernel<F32, kItems>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSmemBytes);
-        attr_set = true;
-    }
+    allow_smem<small_build_kernel<F32, kItems>>(kSmemBytes);
     small_build_kernel<F32, kItems><<<1, kSB, kSmemBytes, s>>>(a);
 }
 

@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kThreads) pass_kernel(const K *__restrict__ ki
 }
 
 template <typename K, int kItems>
-size_t pass_smem()
+constexpr size_t pass_smem()
 {
     return sizeof(unsigned) * (kWarps * kRadix + 2 * kRadix + 16) + (sizeof(K) + sizeof(int)) * kThreads * kItems;
 }
@@ -249,12 +249,8 @@ int sort_impl(K *ka, K *kb, int *va, int *vb, int n, int bits, void *scratch, un
         hb = hb < 1 ? 1 : (hb > 1216 ? 1216 : hb);
         hist_kernel<K><<<hb, kThreads, 0, s>>>(ka, n, npass, hist);
     }
-    static bool attr_set = false;
-    const size_t smem = pass_smem<K, kItems>();
-    if (!attr_set) {
-        cudaFuncSetAttribute(pass_kernel<K, kItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr_set = true;
-    }
+    constexpr size_t smem = pass_smem<K, kItems>();
+    static_assert(smem <= 48 * 1024, "no opt-in needed");
     K *src_k = ka, *dst_k = kb;
     int *src_v = nullptr, *dst_v = vb;
     int *v_first_dst = vb;
@@ -312,7 +308,6 @@ int sort_wait_selftest(int spin_limit, unsigned *err_out, cudaStream_t s)
     const unsigned one = 1u;
     cudaMemcpyAsync(ticket, &one, sizeof one, cudaMemcpyHostToDevice, s);   // the block takes tile 1
     const size_t smem = pass_smem<unsigned, kManyItems>();
-    cudaFuncSetAttribute(pass_kernel<unsigned, kManyItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     pass_kernel<unsigned, kManyItems><<<1, kThreads, smem, s>>>(kin, nullptr, kout, vout, n, 0, base, status, ticket, err,
                                                     spin_limit);   // tile 1: never scans
     cudaMemcpyAsync(err_out, err, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
