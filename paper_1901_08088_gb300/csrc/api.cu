@@ -104,10 +104,14 @@ struct qbvh_ctx {
     DevBuf cell_start, stype;
     DevBuf leaves64;
     DevBuf boxes;
-    DevBuf lj_partials, lj_blk_sys, lj_blk_first, lj_sys_blk;
-    std::vector<int> lj_layout_off;   // offsets the LJ block tables were built for
-    int lj_layout_particles = 0;      // and the particles per block
-    int lj_n_blocks = 0;
+    DevBuf lj_partials;
+    // LJ block tables and records, [k] for blocks of 2^k particles.  The lanes option
+    // chooses the block size, and a recorded launch keeps the one it was made with.
+    struct LJBlocks {
+        DevBuf sys, first, sys_start, partials;
+        std::vector<int> off;   // offsets the tables were built for
+        int n = 0;
+    } lj_blocks[9];
     // uploads cached by content
     std::vector<SysInfo> up_sys;
     std::vector<int> up_off;
@@ -644,9 +648,10 @@ int qbvh_destroy(qbvh_handle h)
                          &h->nodes21,
                          &h->leaves, &h->leaf_q, &h->range, &h->child, &h->par_int, &h->par_leaf, &h->visit,
                          &h->seg, &h->acc, &h->seg_start, &h->frames, &h->sys, &h->sys_off, &h->status,
-                         &h->rows, &h->counts, &h->cell_start, &h->stype, &h->lj_partials, &h->lj_blk_sys, &h->lj_blk_first,
-                         &h->lj_sys_blk, &h->leaves64, &h->boxes};
+                         &h->rows, &h->counts, &h->cell_start, &h->stype, &h->lj_partials, &h->leaves64, &h->boxes};
         for (DevBuf *b : all) release(*b);
+        for (auto &k : h->lj_blocks)
+            for (DevBuf *b : {&k.sys, &k.first, &k.sys_start, &k.partials}) release(*b);
         if (h->h_status) cudaFreeHost(h->h_status);
     }
     delete h;
@@ -858,7 +863,10 @@ int qbvh_lj_forward(qbvh_handle h, const void *pos_dev, const float *eps_dev, co
     const int tpp = !h->lj_tpp_set && lj_spread(h->n) ? 0 : h->lj_tpp;
     const int B = lj_particles_per_block(h->n, tpp);
     int rc = QBVH_OK;
-    if (h->lj_layout_off != h->off || h->lj_layout_particles != B || h->lj_blk_sys.p == nullptr) {
+    int log2_b = 0;
+    while ((1 << log2_b) < B) ++log2_b;
+    auto &blocks = h->lj_blocks[log2_b];
+    if (blocks.off != h->off || blocks.sys.p == nullptr) {
         std::vector<int> blk_sys, blk_first, sys_blk(h->n_sys + 1, 0);
         for (int k = 0; k < h->n_sys; ++k) {
             sys_blk[k] = (int)blk_sys.size();
@@ -868,25 +876,25 @@ int qbvh_lj_forward(qbvh_handle h, const void *pos_dev, const float *eps_dev, co
             }
         }
         sys_blk[h->n_sys] = (int)blk_sys.size();
-        h->lj_n_blocks = (int)blk_sys.size();
+        blocks.n = (int)blk_sys.size();
+        blocks.off.clear();
         if (blk_sys.empty()) {
             blk_sys.push_back(0);
             blk_first.push_back(0);
         }
-        rc = rc ? rc : ensure(h, h->lj_blk_sys, blk_sys.size() * 4);
-        rc = rc ? rc : ensure(h, h->lj_blk_first, blk_first.size() * 4);
-        rc = rc ? rc : ensure(h, h->lj_sys_blk, sys_blk.size() * 4);
+        rc = rc ? rc : ensure(h, blocks.sys, blk_sys.size() * 4);
+        rc = rc ? rc : ensure(h, blocks.first, blk_first.size() * 4);
+        rc = rc ? rc : ensure(h, blocks.sys_start, sys_blk.size() * 4);
         if (rc) return rc;
-        if (cudaMemcpyAsync(h->lj_blk_sys.p, blk_sys.data(), blk_sys.size() * 4, cudaMemcpyHostToDevice, stream) ||
-            cudaMemcpyAsync(h->lj_blk_first.p, blk_first.data(), blk_first.size() * 4, cudaMemcpyHostToDevice,
+        if (cudaMemcpyAsync(blocks.sys.p, blk_sys.data(), blk_sys.size() * 4, cudaMemcpyHostToDevice, stream) ||
+            cudaMemcpyAsync(blocks.first.p, blk_first.data(), blk_first.size() * 4, cudaMemcpyHostToDevice,
                             stream) ||
-            cudaMemcpyAsync(h->lj_sys_blk.p, sys_blk.data(), sys_blk.size() * 4, cudaMemcpyHostToDevice, stream))
+            cudaMemcpyAsync(blocks.sys_start.p, sys_blk.data(), sys_blk.size() * 4, cudaMemcpyHostToDevice, stream))
             return QBVH_ERR_CUDA;
-        h->lj_layout_off = h->off;
-        h->lj_layout_particles = B;
+        blocks.off = h->off;
     }
     const int np = 1 + 2 * T * T;
-    rc = ensure(h, h->lj_partials, (size_t)(h->lj_n_blocks > 0 ? h->lj_n_blocks : 1) * np * 8);
+    rc = ensure(h, blocks.partials, (size_t)(blocks.n > 0 ? blocks.n : 1) * np * 8);
     if (rc) return rc;
     a.pos = reinterpret_cast<const float4 *>(pos_dev);
     a.order = h->lj_zorder ? reinterpret_cast<const int *>(h->vals[h->sorted].p) : nullptr;
@@ -897,20 +905,20 @@ int qbvh_lj_forward(qbvh_handle h, const void *pos_dev, const float *eps_dev, co
     a.n_types = T;
     a.n_sys = h->n_sys;
     a.sys = reinterpret_cast<const SysInfo *>(h->sys.p);
-    a.blk_sys = reinterpret_cast<const int *>(h->lj_blk_sys.p);
-    a.blk_first = reinterpret_cast<const int *>(h->lj_blk_first.p);
-    a.n_blocks = h->lj_n_blocks;
+    a.blk_sys = reinterpret_cast<const int *>(blocks.sys.p);
+    a.blk_first = reinterpret_cast<const int *>(blocks.first.p);
+    a.n_blocks = blocks.n;
     a.particles = B;
     a.tpp = tpp;
     a.eps = eps_dev;
     a.sig = sig_dev;
     a.e = e_dev;
     a.F = F_dev;
-    a.partials = reinterpret_cast<double *>(h->lj_partials.p);
+    a.partials = reinterpret_cast<double *>(blocks.partials.p);
     a.U = U_dev;
     a.dE = dE_dev;
     a.dS = dS_dev;
-    a.sys_blk_start = reinterpret_cast<const int *>(h->lj_sys_blk.p);
+    a.sys_blk_start = reinterpret_cast<const int *>(blocks.sys_start.p);
     launch_lj_forward(a, stream);
     return cuda_status();
 }

@@ -83,3 +83,21 @@ def test_traversal_blocks_keep_the_shared_memory_limit(host, n):
             assert h.build(n) == 0 and h.query() == 0
             h.close()
     assert host.fake_limits_lowered() == before
+
+
+@pytest.mark.parametrize("T", [1, 2])
+def test_lj_tables_outlive_other_lanes(host, T):
+    """A recorded LJ launch reads its block tables and writes its block records on
+    every replay: a pass with other lanes over the same systems leaves both alone."""
+    h = Handle(host)
+    assert h.build(70000, T) == 0 and h.query(T) == 0
+    host.fake_forget_uploads()
+    h.forces(T)
+    frees = host.fake_frees()
+    assert host.fake_uploads() > 0
+    for lanes in (8, 32, 1, 16, 4, 2):
+        h.set("LJ_LANES", lanes)
+        h.forces(T)
+        assert host.fake_uploads_lost() == 0
+        assert host.fake_frees() == frees
+    h.close()
