@@ -74,7 +74,8 @@ __device__ __forceinline__ int4 row_chunk(const int *row, int k, int sub, int c)
 // order, from each other's registers.
 //
 // FP64 runs at about two operations per cycle and SM: an instruction of a warp
-// takes 16 cycles.  Lane 0 of a particle adds up its dU/deps terms and lane 1 its
+// takes 16 cycles.  Every lane's FP32 sums of gradient terms enter FP64 by
+// themselves: even lanes add up the particle's dU/deps terms and odd ones its
 // dU/dsig terms, in the same instructions.  GRAD = false leaves them out where
 // the caller asked for neither.
 template <int T, int TPP, bool GRAD, bool SPREAD>
@@ -85,6 +86,11 @@ lj_forward_kernel(const __grid_constant__ LJArgs a)
     constexpr int NP = 1 + 2 * T * T;
     constexpr int TG = GRAD ? T : 1;
     constexpr int SETS = TPP == 1 ? 2 : 1;   // one lane keeps both gradients' sums
+    // lanes of a particle that keep FP64 sums: its other lanes add to theirs in every
+    // round, or (16 and 32 lanes, where that is four and five more additions a round) all
+    // lanes keep their own to the end.  Two types, N = 300,000, 4 / 8 / 16 / 32 lanes:
+    // 149 / 184 / 252 / 422 us the first way, 153 / 182 / 231 / 317 the second.
+    constexpr int KEEP = TPP <= 8 ? (TPP == 1 ? 1 : 2) : TPP;
     __shared__ LJParams s_par[T * T];
     __shared__ double s_red[kLJBlock / 32][NP];
     const int tid = threadIdx.x;
@@ -179,13 +185,6 @@ lj_forward_kernel(const __grid_constant__ LJArgs a)
             fx += __shfl_xor_sync(0xFFFFFFFFu, fx, o);
             fy += __shfl_xor_sync(0xFFFFFFFFu, fy, o);
             fz += __shfl_xor_sync(0xFFFFFFFFu, fz, o);
-            if (GRAD) {
-#pragma unroll
-                for (int b = 0; b < TG; ++b) {
-                    gE[b] += __shfl_xor_sync(0xFFFFFFFFu, gE[b], o);
-                    gS[b] += __shfl_xor_sync(0xFFFFFFFFu, gS[b], o);
-                }
-            }
         }
         if (i >= 0 && sub == 0) {
             if (a.e) a.e[i] = 0.5f * ei;
@@ -196,17 +195,20 @@ lj_forward_kernel(const __grid_constant__ LJArgs a)
             }
         }
         // FP64 sums of the energy (a lane's FP32 sum; SPREAD: lanes 0 and 4 hold the
-        // two) and of the parameter-gradient terms; the factor 1/2 comes at the end
+        // two) and of the lanes' parameter-gradient terms; the factor 1/2 comes at the end
         if (!SPREAD || (sub & 3) == 0) v += (double)e;
-        if (GRAD && sub < 2) {
+        if (GRAD) {
 #pragma unroll
             for (int h = 0; h < SETS; ++h) {
 #pragma unroll
                 for (int b = 0; b < TG; ++b) {
-                    const double g = (double)((TPP == 1 ? h == 1 : sub == 1) ? gS[b] : gE[b]);
+                    double g = (double)((TPP == 1 ? h == 1 : (sub & 1) != 0) ? gS[b] : gE[b]);
+                    if (TPP > 1) g += (double)__shfl_xor_sync(0xFFFFFFFFu, (sub & 1) ? gE[b] : gS[b], 1);
+#pragma unroll
+                    for (int o = TPP / 2; TPP > 1 && o >= KEEP; o >>= 1) g += __shfl_xor_sync(0xFFFFFFFFu, g, o);
 #pragma unroll
                     for (int t = 0; t < TG; ++t)
-                        if (t == ta) acc[h][t * TG + b] += g;
+                        if (t == ta && sub < KEEP) acc[h][t * TG + b] += g;
                 }
             }
         }
@@ -222,7 +224,7 @@ lj_forward_kernel(const __grid_constant__ LJArgs a)
             for (int q = 0; q < TG * TG; ++q) {
                 double x = acc[h][q];
 #pragma unroll
-                for (int o = 16; o >= TPP; o >>= 1) x += __shfl_down_sync(0xFFFFFFFFu, x, o);
+                for (int o = 16; o >= (KEEP < TPP || TPP == 1 ? TPP : 2); o >>= 1) x += __shfl_down_sync(0xFFFFFFFFu, x, o);
                 // lane 0: dU/deps; lane 1 (one lane per particle: the second set): dU/dsig
                 if (TPP == 1 ? lane == 0 : lane < 2) s_red[warp][(1 + (TPP == 1 ? h : lane) * T * T + q) % NP] = x;
             }

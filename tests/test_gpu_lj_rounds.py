@@ -49,3 +49,58 @@ def test_rounds(n, T, lanes, grad):
         assert np.allclose(dE.cpu().numpy(), ref["dE"], rtol=1e-5, atol=0)
         assert np.allclose(dS.cpu().numpy(), ref["dS"], rtol=1e-5, atol=0)
     nl.close()
+
+
+def _pass(nl, pos4, T, r_cut):
+    """U, dU/deps, dU/dsig of the handle's systems with every eps and sigma one."""
+    S = nl.n_sys
+    one = torch.ones((T, T), device="cuda")
+    U = torch.empty(S, device="cuda", dtype=torch.float64)
+    dE, dS = (torch.empty((S, T, T), device="cuda", dtype=torch.float64) for _ in range(2))
+    check(qbvh_lj_forward(nl.h, pos4, one, one, np.full((T, T), r_cut, np.float32), None, U, None, dE, dS),
+          "qbvh_lj_forward")
+    return U.cpu().numpy(), dE.cpu().numpy(), dS.cpu().numpy()
+
+
+@pytest.mark.parametrize("lanes", [None, 1, 2, 4, 8, 16, 32])
+def test_gradient_terms_enter_fp64_per_lane(lanes):
+    """With eps = 1 a lane's FP32 sum of dU/deps terms is its FP32 sum of energies,
+    so both FP64 totals add the same numbers: equal up to FP64 roundings (32,768
+    particles of up to 32 lanes, sums of one sign: 1e-12).  One FP32 rounding per
+    particle on the way would show as about 2^-24 / sqrt(32,768) = 3e-10."""
+    n, r_cut = 32768, np.float32(2.5)
+    rng = np.random.default_rng(4)
+    ijk = np.stack(np.meshgrid(*[np.arange(32)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    x = ((ijk + 0.5) * 1.1 + 0.08 * rng.uniform(-1, 1, (n, 3))).astype(np.float32)
+    pos4 = torch.from_numpy(np.concatenate([x, np.zeros((n, 1), np.float32)], 1)).cuda()
+    nl = NeighborList()
+    if lanes is not None:
+        nl.set_option(_lib.QBVH_OPT_LJ_LANES, lanes)
+    nl.build(pos4, 35.2, 1).query(float(r_cut), cap=96)
+    U, dE, _ = _pass(nl, pos4, 1, r_cut)
+    nl.close()
+    assert abs(dE[0, 0, 0] - U[0]) <= 1e-12 * abs(U[0])
+
+
+@pytest.mark.parametrize("T", [1, 2, 3])
+def test_gradient_terms_of_a_cluster(T):
+    """Nine particles in reach of one another: with eight lanes per particle every
+    lane holds one pair, so the totals are those of the 36 pairs, each computed as a
+    system of its own, added in FP64 (36 terms: 1e-14 of their sizes)."""
+    rng = np.random.default_rng(8)
+    g = np.stack(np.meshgrid(*[np.arange(3)] * 2, indexing="ij"), -1).reshape(-1, 2)
+    x = np.concatenate([g, np.zeros((9, 1))], 1) * 1.05 + 0.08 * rng.uniform(-1, 1, (9, 3)) + 9.0
+    t = rng.integers(0, T, 9).astype(np.int32)
+    p = np.concatenate([x.astype(np.float32), t.view(np.float32)[:, None]], 1)
+    i, j = np.triu_indices(9, 1)
+    pairs = np.stack([p[i], p[j]], 1).reshape(-1, 4)
+    got = []
+    for q, S in ((p, 1), (pairs, 36)):
+        q = torch.from_numpy(np.ascontiguousarray(q)).cuda()
+        nl = NeighborList()
+        nl.build_batched(q, np.arange(S + 1) * (len(q) // S), [20.0] * S, T).query(4.0, cap=8)
+        assert int(nl.neighbors()[1].min()) == (8 if S == 1 else 1)
+        got.append(_pass(nl, q, T, np.float32(4.0))[1:])
+        nl.close()
+    for whole, parts in zip(*got):
+        assert np.all(np.abs(whole[0] - parts.sum(0)) <= 1e-14 * np.abs(parts).sum(0))
