@@ -110,9 +110,9 @@ int qbvh_destroy(qbvh_handle h);
  * every build writes.  Takes effect at the next build. */
 #define QBVH_OPT_NODE_FORMAT 5
 /* Lanes that share one particle's row in qbvh_lj_forward: 1, 2, 4, 8, 16 or
- * 32 (default 2).  More lanes read a row in longer contiguous chunks.  Until
- * the option is set, small systems take 8 lanes that form the same FP32 sums
- * as 2 do. */
+ * 32 (default 2).  More lanes read a row in longer contiguous chunks.  With 2,
+ * lists of fewer than 30,000 particles take 8 lanes that form the same FP32
+ * energy sums as 2 do. */
 #define QBVH_OPT_LJ_LANES 6
 /* 1 (default): qbvh_lj_forward visits particles in the Z-order of the last
  * build (neighbouring particles share cached positions); 0: original order.

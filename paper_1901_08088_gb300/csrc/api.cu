@@ -68,8 +68,7 @@ struct qbvh_ctx {
     int traversal = 1;
     int warp_particles = 32;
     int node_fmt = 0;      // 0: 10-bit quantized nodes (Fig. 3b), 1: FP32 nodes (Fig. 3a), 2: 21-bit nodes
-    int lj_tpp = 2;        // lanes per particle in the LJ pass (few particles: lj_spread, unless the caller set them)
-    bool lj_tpp_set = false;
+    int lj_tpp = 2;        // lanes per particle in the LJ pass (2: few particles take lj_spread)
     int lj_zorder = 1;     // LJ pass walks particles in the tree's Z-order
     int method = 0;        // 0: quantized BVH, 1: uniform grid comparator
     int grid_tpp = 8;      // lanes per particle of the grid traversal
@@ -685,7 +684,6 @@ int qbvh_set_option(qbvh_handle h, int option, int value)
     case QBVH_OPT_LJ_LANES:
         if (value < 1 || value > 32 || (value & (value - 1))) return QBVH_ERR_INVALID_ARG;
         h->lj_tpp = value;
-        h->lj_tpp_set = true;
         return QBVH_OK;
     case QBVH_OPT_LJ_ZORDER:
         if (value != 0 && value != 1) return QBVH_ERR_INVALID_ARG;
@@ -860,7 +858,7 @@ int qbvh_lj_forward(qbvh_handle h, const void *pos_dev, const float *eps_dev, co
     }
     DeviceGuard g(h->device);
     // block tables: every block covers particles of one system
-    const int tpp = !h->lj_tpp_set && lj_spread(h->n) ? 0 : h->lj_tpp;
+    const int tpp = h->lj_tpp == 2 && lj_spread(h->n) ? 0 : h->lj_tpp;
     const int B = lj_particles_per_block(h->n, tpp);
     int rc = QBVH_OK;
     int log2_b = 0;

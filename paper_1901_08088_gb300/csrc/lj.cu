@@ -316,8 +316,8 @@ int lj_particles_per_block(int n, int tpp)
     return p;
 }
 
-// 8 lanes per particle where the caller has not chosen them and two would leave
-// most of the GPU idle: two-type gradients of 2 x 2827 particles 29 -> 19 us,
+// 8 lanes per particle that keep the sums of two, where two (the default) would
+// leave most of the GPU idle: two-type gradients of 2 x 2827 particles 29 -> 19 us,
 // N = 30,011 33 us either way, N = 131,072 with r = 1.12 27 -> 50 us.
 bool lj_spread(int n) { return n < 30000; }
 

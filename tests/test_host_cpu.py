@@ -101,3 +101,19 @@ def test_lj_tables_outlive_other_lanes(host, T):
         assert host.fake_uploads_lost() == 0
         assert host.fake_frees() == frees
     h.close()
+
+
+@pytest.mark.parametrize("n", [100, 20000, 70000])
+def test_writing_an_option_back_changes_nothing(host, n):
+    """The default of the LJ lanes is the value that get_option returns and that the
+    autotuner starts from: setting it leaves the kernel of a pass the same."""
+    from paper_1901_08088_gb300.autotune import DEFAULTS
+
+    h = Handle(host)
+    assert h.build(n) == 0 and h.query() == 0
+    kernels = h.forces()
+    assert DEFAULTS[_lib.QBVH_OPT_LJ_LANES] == h.get("LJ_LANES")
+    assert h.set("LJ_LANES", 8) == 0 and h.forces() != kernels
+    assert h.set("LJ_LANES", DEFAULTS[_lib.QBVH_OPT_LJ_LANES]) == 0
+    assert h.forces() == kernels
+    h.close()
