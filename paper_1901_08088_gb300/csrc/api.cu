@@ -547,6 +547,7 @@ int query_enqueue(qbvh_ctx *h, const float *r_list_host, int cap, cudaStream_t s
     q.rows = reinterpret_cast<int *>(h->rows.p);
     q.counts = reinterpret_cast<int *>(h->counts.p);
     q.status = st;
+    q.spread = reinterpret_cast<int *>(h->visit.p);   // the fit's arrival counters: free until the next build
     q.candidates = h->candidates;
     q.traversal = h->traversal;
     q.warp_particles = h->warp_particles;

@@ -502,6 +502,7 @@ struct QueryArgs {
     float rl2_hi[64];
     double r2_64[64];
     int block;
+    int *spread;           // [n / 32, rounded up] marks of spread runs (query_wide.cu)
     int sparse_blocks;     // leading blocks that walk sparse trees one particle per warp
     float r_list[64];      // [a][b] list radius
     float rl2[64];         // fl(r * r)

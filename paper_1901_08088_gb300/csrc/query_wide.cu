@@ -522,7 +522,7 @@ __device__ __forceinline__ int row_index(const QueryArgs &a, int s, const float4
 
 // one particle by the whole warp (W = 32)
 template <bool F64>
-__device__ __forceinline__ void walk_particle(const QueryArgs &a, int s, int seg, int T)
+__device__ __forceinline__ int walk_particle(const QueryArgs &a, int s, int seg, int T)
 {
     const float4 me = __ldg(a.leaves + s);
     const int i = row_index(a, s, me);
@@ -536,7 +536,7 @@ __device__ __forceinline__ void walk_particle(const QueryArgs &a, int s, int seg
     const int sys = seg / T;
     walk_trees<F64, 32>(a, c, out, nullptr, w, sys, seg - sys * T, T, true, false, -1, 0, 0);
     if ((threadIdx.x & 31) == 0) a.counts[i] = out.count;
-    warp_max_count(out.count, a.status);
+    return out.count;
 }
 
 // the leading blocks: every particle of a sparse tree (query_common.cuh) gets a warp
@@ -547,7 +547,123 @@ __device__ __forceinline__ void sparse_walks(const QueryArgs &a)
     for (int ta = 0; ta < a.n_types; ++ta) {
         if (!sparse_tree(a, ta)) continue;
         const int start = a.seg[ta].start, count = a.seg[ta].count;
-        for (int p = gw; p < count; p += nw) walk_particle<false>(a, start + p, ta, a.n_types);
+        for (int p = gw; p < count; p += nw) warp_max_count(walk_particle<false>(a, start + p, ta, a.n_types), a.status);
+    }
+}
+
+// ---- spread packets --------------------------------------------------------
+// The boxes around far-apart particles (a dilute type among a dense one, vapor around
+// a droplet) cover most of the system, and the packet's warp would test most of its
+// leaves, alone and long after the others.  Spread is a run of 32 leaves whose boxes
+// (box1[run], grown by the radius) cover more than kSpreadVolume times what the cubes
+// around 32 separate spheres do and reach more than kSpreadChunks chunks of leaves
+// under the zero image: a gas stays with its packets, which find little.
+// spread_kernel marks these runs and walks their particles one per warp; the packets'
+// walk passes over them.  The rows are the same either way.
+//
+// Query, milliseconds, walk of the binary tree / packets alone / this: 64 particles of
+// a second type among 2,000,000 in double precision 5.1 / 28.9 / 1.9; four types of 64
+// among 2,000,000 of a fifth 4.1 / 27.2 / 1.7; four batched systems of 250,000 with 32
+// each 3.3 / 5.9 / 0.85; a droplet of 1,000,000 with 100,000 vapor particles in a box
+// of 4000, radius 1.2, 1.07 / 1.61 / 0.35.  It costs 2 to 4 us per query (N = 30,011 58 ->
+// 61, 131,072 with r = 1.42 65 -> 67, 2,097,152 953 -> 959), and a gas of 1,000,000 at
+// density 0.0005 the counting of its chunks, 119 -> 167 us (binary tree 224).
+//
+// Four times: up to there a packet tests at most about 30,000 leaves at density 0.8
+// and radius 3.3, fewer than the walk of the binary tree did (44,000).  128 chunks are
+// four per particle: a particle by itself visits 20 to 25 there.
+constexpr float kSpreadVolume = 4.f;
+constexpr int kSpreadChunks = 128;
+constexpr int kSpreadRuns = 8;   // most runs per warp of spread_kernel
+
+__device__ __forceinline__ int chunks_reached(const QueryArgs &a, int first, int last, const Packet &p, float rs2, int n)
+{
+    for (int n3 = first >> 15; n3 <= last >> 15; n3 += 32) {
+        unsigned M3 = test_boxes(a.box3, n3, first >> 15, last >> 15, p, rs2);
+        while (M3) {
+            const int c3 = (n3 + __ffs(M3) - 1) << 5;
+            M3 &= M3 - 1u;
+            unsigned M2 = test_boxes(a.box2, c3, first >> 10, last >> 10, p, rs2);
+            while (M2) {
+                n += __popc(test_boxes(a.box1, (c3 + __ffs(M2) - 1) << 5, first >> 5, last >> 5, p, rs2));
+                if (n > kSpreadChunks) return n;
+                M2 &= M2 - 1u;
+            }
+        }
+    }
+    return n;
+}
+
+__device__ __forceinline__ int seg_of_leaf(const QueryArgs &a, int s)
+{
+    return a.wide_keys ? seg_of_sorted<true>(a, s) : seg_of_sorted<false>(a, s);
+}
+
+__device__ __forceinline__ Box box_of_lane(const Box &b, int src)
+{
+    return Box{__shfl_sync(FULL, b.lx, src), __shfl_sync(FULL, b.ly, src), __shfl_sync(FULL, b.lz, src),
+               __shfl_sync(FULL, b.hx, src), __shfl_sync(FULL, b.hy, src), __shfl_sync(FULL, b.hz, src)};
+}
+
+// Comes before the packets' walk.  A block takes every gridDim.x-th run, `runs` per
+// warp (spread ones lie side by side), and shares the particles of the spread ones it
+// finds among its warps.
+template <bool F64>
+__global__ void __launch_bounds__(256, 4) spread_kernel(const __grid_constant__ QueryArgs a, int runs)
+{
+    __shared__ int s_run[8 * kSpreadRuns];
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, T = a.n_types;
+    const long long run = ((threadIdx.x >> 5) * runs + lane) * (long long)gridDim.x + blockIdx.x;
+    bool wide = false;
+    int seg = 0;
+    Packet p{};
+    if (lane < runs && 32 * run < a.n) {
+        seg = seg_of_leaf(a, 32 * (int)run);   // of the run's first particle
+        const int ta = seg % T;
+        float rs = 0.f;
+        for (int tb = 0; tb < T; ++tb) rs = fmaxf(rs, a.r_list[ta * T + tb] > 0.f ? a.rs[ta * T + tb] : 0.f);
+        float4 b[4];
+        node32_ld(a.box1 + 4 * run, b[0], b[1]);
+        node32_ld(a.box1 + 4 * run + 2, b[2], b[3]);
+        p.a = Box{b[0].x, b[0].y, b[0].z, b[0].w, b[1].x, b[1].y};
+        p.b = Box{b[2].x, b[2].y, b[2].z, b[2].w, b[3].x, b[3].y};
+        const float d = 2.f * rs;
+        // (an empty side has lower corners of +inf; a sparse tree has its own walk)
+        wide = grown_volume(p.a, d) + (p.b.lx <= p.b.hx ? grown_volume(p.b, d) : 0.f) > kSpreadVolume * 32.f * d * d * d &&
+               !(!F64 && a.sparse_blocks > 0 && sparse_tree(a, seg));
+    }
+    bool mark = false;
+    unsigned todo = __ballot_sync(FULL, wide);
+    while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int sg = __shfl_sync(FULL, seg, src), sys = sg / T, ta = sg - sys * T;
+        const Packet q{box_of_lane(p.a, src), box_of_lane(p.b, src), true};
+        int n = 0;
+        for (int tb = 0; tb < T && n <= kSpreadChunks; ++tb) {
+            const SegInfo &g = a.seg[sys * T + tb];
+            if (a.r_list[ta * T + tb] > 0.f && g.count > 0)
+                n = chunks_reached(a, g.start, g.start + g.count - 1, q, a.rs2[ta * T + tb], n);
+        }
+        if (lane == src) mark = n > kSpreadChunks;
+    }
+    if (lane < runs && 32 * run < a.n) {
+        a.spread[run] = mark;
+        if (mark) s_run[atomicAdd(&s_n, 1)] = (int)run;
+    }
+    __syncthreads();
+    // (at the start, the walk's blocks would be placed around this kernel's: N = 30,011
+    // 72 us instead of 62)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int k = threadIdx.x >> 5; k < 32 * s_n; k += 8) {
+        const int s = 32 * s_run[k >> 5] + (k & 31);
+        if (s >= a.n) continue;
+        const int sg = seg_of_leaf(a, s);
+        if (!F64 && a.sparse_blocks > 0 && sparse_tree(a, sg)) continue;
+        warp_max_count(walk_particle<F64>(a, s, sg, T), a.status);
     }
 }
 
@@ -560,6 +676,8 @@ template <bool ONE, bool F64, int W>
 __global__ void __launch_bounds__(256, W == 1 && !(ONE && F64) ? 3 : 4) wide_query_kernel(const __grid_constant__ QueryArgs a)
 {
     constexpr int G = 32 / W;
+    // (double-precision data: waiting here took 8 us more than a plain launch, N = 131,072)
+    if (W < 32 && !F64) pdl_begin();
     int blk = (int)blockIdx.x, nblk = (int)gridDim.x;
     const bool sparse = !ONE && !F64 && a.sparse_blocks > 0;
     if (sparse) {
@@ -581,9 +699,13 @@ __global__ void __launch_bounds__(256, W == 1 && !(ONE && F64) ? 3 : 4) wide_que
     const int seg_i = !active ? -1 : (ONE ? 0 : (a.wide_keys ? seg_of_sorted<true>(a, s) : seg_of_sorted<false>(a, s)));
     if (W == 32) {
         if (!active || (sparse && sparse_tree(a, seg_i))) return;
-        walk_particle<F64>(a, s, seg_i, T);
+        warp_max_count(walk_particle<F64>(a, s, seg_i, T), a.status);
         return;
     }
+    // walked by spread_kernel (a single tree leaves here, others pass over their trees:
+    // one return too many cost 32 x 65,536 particles 6 us, one flag too many 8 at 2,097,152)
+    const bool marked = packet * G < a.n && __ldcg(a.spread + ((packet * G) >> 5)) != 0;
+    if (ONE && marked) return;
     const float4 me = active ? __ldg(a.leaves + s) : make_float4(0.f, 0.f, 0.f, 0.f);
     const int i = active ? row_index(a, s, me) : 0;
     unsigned code = 0u;   // 30-bit Z-order code
@@ -599,9 +721,9 @@ __global__ void __launch_bounds__(256, W == 1 && !(ONE && F64) ? 3 : 4) wide_que
     Walk w{0, 0, 0, -1};
     extern __shared__ __align__(16) unsigned char smem[];
     WideStage<W> *st = reinterpret_cast<WideStage<W> *>(smem) + (threadIdx.x >> 5);
-    bool elsewhere = false;   // particle of a sparse tree: walked by the leading blocks
+    bool elsewhere = !ONE && marked;   // or particle of a sparse tree: walked by the leading blocks
     // the warp's particles may belong to several trees: one tree at a time
-    unsigned remaining = __ballot_sync(FULL, active);
+    unsigned remaining = __ballot_sync(FULL, active && !elsewhere);
     while (remaining) {
         const int seg = ONE ? 0 : __shfl_sync(FULL, seg_i, __ffs(remaining) - 1);
         const bool part = ONE ? active : (active && seg_i == seg);
@@ -638,7 +760,17 @@ void launch_w(const QueryArgs &a, int extra, cudaStream_t s)
     const size_t smem = warps * stage_size<W>();
     // blocks of 224 and 256 threads exceed the 48 KB that need no opt-in
     if (smem > 48 * 1024) allow_smem<wide_query_kernel<ONE, F64, W>>(8 * stage_size<W>());
-    wide_query_kernel<ONE, F64, W><<<grid, a.block, smem, s>>>(a);
+    if (W == 32) {
+        wide_query_kernel<ONE, F64, W><<<grid, a.block, smem, s>>>(a);
+        return;
+    }
+    // few runs per warp while the grid is one wave: a gas counts them one after another
+    const int total = (a.n + 31) / 32;
+    int runs = 1;
+    while (runs < kSpreadRuns && total > 8 * runs * 608) runs *= 2;
+    spread_kernel<F64><<<(total + 8 * runs - 1) / (8 * runs), 256, 0, s>>>(a, runs);
+    if (F64) wide_query_kernel<ONE, F64, W><<<grid, a.block, smem, s>>>(a);
+    else launch_pdl(wide_query_kernel<ONE, F64, W>, grid, a.block, smem, s, a);
 }
 
 template <bool F64>
