@@ -161,6 +161,10 @@ __global__ void __launch_bounds__(kBlock) morton_kernel(const BuildArgs a, unsig
             }
             ph = make_float3(p.x, p.y, p.z);
         }
+        // -0 is a coordinate 0: its bits, as an unsigned number the largest, would be the
+        // root box's upper corner
+        p = make_float4(p.x + 0.f, p.y + 0.f, p.z + 0.f, 0.f);
+        ph = make_float3(ph.x + 0.f, ph.y + 0.f, ph.z + 0.f);
         const unsigned code = (spread10(bin_of(p.x, sy.mscale)) << 2) |
                               (spread10(bin_of(p.y, sy.mscale)) << 1) |
                               spread10(bin_of(p.z, sy.mscale));

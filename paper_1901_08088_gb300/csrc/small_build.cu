@@ -120,6 +120,10 @@ __global__ void __launch_bounds__(kSB, 1) small_build_kernel(const BuildArgs a)
                 if (!(p.y == p.y)) p.y = 0.f;
                 if (!(p.z == p.z)) p.z = 0.f;
             }
+            // -0 is a coordinate 0 (as in the Morton pass of build.cu)
+            p.x += 0.f;
+            p.y += 0.f;
+            p.z += 0.f;
             const unsigned code = (spread10(bin_of(p.x, sy.mscale)) << 2) | (spread10(bin_of(p.y, sy.mscale)) << 1) |
                                   spread10(bin_of(p.z, sy.mscale));
             if (T == 1) type = 0;   // every type in the system's one tree

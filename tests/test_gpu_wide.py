@@ -215,3 +215,29 @@ def test_a_dilute_type_costs_little():
         best.append(min(ms))
         nl.close()
     assert best[1] <= 3.0 * best[0]
+
+
+@pytest.mark.parametrize("n", [700, 5000, 20000, 65000])
+@pytest.mark.parametrize("f64", [False, True])
+def test_negative_zero(n, f64):
+    """A coordinate of -0 is the coordinate 0."""
+    x, L = _fluid(n, 0.6, n)
+    x[:40, 0] = 0.0
+    x[20:60, 1] = 0.0
+    rows = []
+    for sign in (1.0, -1.0):
+        y = np.where(x == 0, np.float32(sign * 0.0), x)
+        assert np.signbit(y).any() == (sign < 0)
+        for traversal in (0, 1):
+            nl = NeighborList()
+            nl.set_option(_lib.QBVH_OPT_TRAVERSAL, traversal)
+            if f64:
+                nl.build_f64(torch.from_numpy(np.concatenate([y, np.zeros((n, 1))], 1)).cuda(), L, 1)
+            else:
+                nl.build(_pos4(y), L, 1)
+            nl.query(min(2.2, 0.45 * L), cap=96)
+            r, c = nl.neighbors()
+            rows.append(torch.where(torch.arange(r.shape[1], device="cuda")[None, :] < c[:, None], r, -1))
+            nl.close()
+    for r in rows[1:]:
+        assert torch.equal(r, rows[0])
