@@ -295,11 +295,13 @@ __global__ void __launch_bounds__(1024) seg_scan_kernel(const BuildArgs a, const
     }
 }
 
+// (ordinary loads: the sort's last pass may still run when the hierarchy pass starts,
+// and only they are ordered after pdl_begin)
 template <bool WIDE>
 __device__ __forceinline__ unsigned long long key_at(const void *keys, int k)
 {
-    if (WIDE) return __ldg(reinterpret_cast<const unsigned long long *>(keys) + k);
-    return __ldg(reinterpret_cast<const unsigned *>(keys) + k);
+    if (WIDE) return reinterpret_cast<const unsigned long long *>(keys)[k];
+    return reinterpret_cast<const unsigned *>(keys)[k];
 }
 
 template <bool WIDE>

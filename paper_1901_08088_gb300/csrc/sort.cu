@@ -97,10 +97,11 @@ __device__ __forceinline__ unsigned block_excl_scan256(unsigned v, unsigned *s_w
     return before + x - v;
 }
 
+// (no __restrict__: it would make the input's loads ones of read-only data, and the
+// pass before, which writes it, may still run when this one starts)
 template <typename K, int kItems>
-__global__ void __launch_bounds__(kThreads) pass_kernel(const K *__restrict__ kin, const int *__restrict__ vin,
-                                                        K *__restrict__ kout, int *__restrict__ vout, int n,
-                                                        int shift, const unsigned *__restrict__ bucket_base,
+__global__ void __launch_bounds__(kThreads) pass_kernel(const K *kin, const int *vin, K *kout, int *vout, int n,
+                                                        int shift, const unsigned *bucket_base,
                                                         unsigned *status, unsigned *ticket, unsigned *err,
                                                         int spin_limit)
 {
