@@ -820,9 +820,7 @@ struct LJCtx {
 // lane's particle.
 template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivor_vals(const Query &c, Row &out, const f32x2 X, const f32x2 Y, const f32x2 Z,
-                                              const int2 id, bool on, bool staged, const LJCtx &lj,
-                                              const QueryArgs *A = nullptr, const BundleStage *st = nullptr,
-                                              int t = 0)
+                                              const int2 id, bool on, bool staged, const LJCtx &lj)
 {
     f32x2 dx = f2_sub(X, f2_pack(c.xi, c.xi)), dy = f2_sub(Y, f2_pack(c.yi, c.yi)),
           dz = f2_sub(Z, f2_pack(c.zi, c.zi));
@@ -837,9 +835,8 @@ __device__ __forceinline__ void survivor_vals(const Query &c, Row &out, const f3
     f2_unpack(f2_mul(dz, dz), sz0, sz1);
     const float d0 = __fadd_rn(__fadd_rn(sx0, sy0), sz0);
     const float d1 = __fadd_rn(__fadd_rn(sx1, sy1), sz1);
-    bool a0, a1;
-    a0 = on && d0 < c.rl2 && (!SELF || id.x != c.self_id);
-    a1 = on && d1 < c.rl2 && (!SELF || id.y != c.self_id);
+    const bool a0 = on && d0 < c.rl2 && (!SELF || id.x != c.self_id);
+    const bool a1 = on && d1 < c.rl2 && (!SELF || id.y != c.self_id);
     if (LJ) {
         f32x2 vx = dx, vy = dy, vz = dz;
         float r0 = d0, r1 = d1;
@@ -868,12 +865,12 @@ __device__ __forceinline__ void survivor_vals(const Query &c, Row &out, const f3
 // survivors t, t + 1 of the stage (8-byte loads)
 template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivor_pair(const Query &c, Row &out, int t, bool on, const BundleStage *st,
-                                              bool staged, const LJCtx &lj = LJCtx{}, const QueryArgs *A = nullptr)
+                                              bool staged, const LJCtx &lj = LJCtx{})
 {
     survivor_vals<SHIFT, SELF, LJ>(c, out, *reinterpret_cast<const f32x2 *>(st->x + t),
                                         *reinterpret_cast<const f32x2 *>(st->y + t),
                                         *reinterpret_cast<const f32x2 *>(st->z + t),
-                                        *reinterpret_cast<const int2 *>(st->id + t), on, staged, lj, A, st, t);
+                                        *reinterpret_cast<const int2 *>(st->id + t), on, staged, lj);
 }
 
 // survivors t .. t + 3 of the stage, t a multiple of 4 (16-byte loads; each
@@ -884,16 +881,16 @@ __device__ __forceinline__ void survivor_pair(const Query &c, Row &out, int t, b
 #endif
 template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivor_quad(const Query &c, Row &out, int t, bool on, const BundleStage *st,
-                                              const LJCtx &lj, const QueryArgs *A = nullptr)
+                                              const LJCtx &lj)
 {
     const float4 X = *reinterpret_cast<const float4 *>(st->x + t);
     const float4 Y = *reinterpret_cast<const float4 *>(st->y + t);
     const float4 Z = *reinterpret_cast<const float4 *>(st->z + t);
     const int4 I = *reinterpret_cast<const int4 *>(st->id + t);
     survivor_vals<SHIFT, SELF, LJ>(c, out, f2_pack(X.x, X.y), f2_pack(Y.x, Y.y), f2_pack(Z.x, Z.y),
-                                        make_int2(I.x, I.y), on, true, lj, A, st, t);
+                                        make_int2(I.x, I.y), on, true, lj);
     survivor_vals<SHIFT, SELF, LJ>(c, out, f2_pack(X.z, X.w), f2_pack(Y.z, Y.w), f2_pack(Z.z, Z.w),
-                                        make_int2(I.z, I.w), on, true, lj, A, st, t + 2);
+                                        make_int2(I.z, I.w), on, true, lj);
 }
 
 // Every lane tests every survivor (one particle per lane), two per step: the
@@ -906,25 +903,25 @@ __device__ __forceinline__ void survivor_quad(const Query &c, Row &out, int t, b
 // completed sectors written once per 8 survivors and at the end.
 template <bool SHIFT, bool SELF, bool LJ = false>
 __device__ __forceinline__ void survivors_loop(const Query &c, Row &out, int s, bool on, const BundleStage *st,
-                                               const LJCtx &lj = LJCtx{}, const QueryArgs *A = nullptr)
+                                               const LJCtx &lj = LJCtx{})
 {
     const bool staged = out.ring != nullptr;
     int t = 0;
     if (staged) {
         for (; t + 8 <= s; t += 8) {
 #if QBVH_SURVIVOR_QUAD
-            survivor_quad<SHIFT, SELF, LJ>(c, out, t, on, st, lj, A);
-            survivor_quad<SHIFT, SELF, LJ>(c, out, t + 4, on, st, lj, A);
+            survivor_quad<SHIFT, SELF, LJ>(c, out, t, on, st, lj);
+            survivor_quad<SHIFT, SELF, LJ>(c, out, t + 4, on, st, lj);
 #else
-            survivor_pair<SHIFT, SELF, LJ>(c, out, t, on, st, true, lj, A);
-            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 2, on, st, true, lj, A);
-            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 4, on, st, true, lj, A);
-            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 6, on, st, true, lj, A);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t, on, st, true, lj);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 2, on, st, true, lj);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 4, on, st, true, lj);
+            survivor_pair<SHIFT, SELF, LJ>(c, out, t + 6, on, st, true, lj);
 #endif
             out.check();
         }
     }
-    for (; t + 1 < s; t += 2) survivor_pair<SHIFT, SELF, LJ>(c, out, t, on, st, staged, lj, A);
+    for (; t + 1 < s; t += 2) survivor_pair<SHIFT, SELF, LJ>(c, out, t, on, st, staged, lj);
     if (t < s) {
         const float4 q = make_float4(st->x[t], st->y[t], st->z[t], 0.f);
         const int id = st->id[t];
@@ -1108,7 +1105,7 @@ __device__ __forceinline__ void bundle_filtered(const QueryArgs &a, const Query 
     }
     s += pad;
     __syncwarp();
-    if (W == 1) survivors_loop<SHIFT, SELF, LJ>(c, out, s, on, st, lj, &a);
+    if (W == 1) survivors_loop<SHIFT, SELF, LJ>(c, out, s, on, st, lj);
     else survivors_loop_w<SHIFT, SELF, W>(c, out, s, on, st, wsub, same);
     __syncwarp();   // the next bundle rewrites the stage
 }
