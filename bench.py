@@ -114,6 +114,8 @@ PROFILED_TRAFFIC = {
 # scan, 4 onesweep passes (30-bit keys, 8-bit digits), Karras, fit; query = 1
 # traversal launch (all periodic images); LJ = forward + fixed-order FP64 finalize
 KERNELS_PER_STEP = 9 + 1 + 2
+# before the traversal of the default mapping: the pass that marks spread packets
+KERNELS_SPREAD = 1
 # with the LJ terms summed inside the traversal: build, traversal, finalize
 KERNELS_PER_STEP_FUSED = 9 + 1 + 1
 _TRAFFIC_SOURCES = ("paper_1901_08088_gb300/csrc/query_wide.cu", "paper_1901_08088_gb300/csrc/query_common.cuh",
@@ -340,9 +342,11 @@ def run_ours(args):
     s_build, t_query, t_lj = split_times(max(5, min(args.steps, 20)))
 
     # build and query under each node format (the tuned options otherwise):
-    # the paper's 10-bit quantized nodes (Fig. 3b) and FP32 nodes (Fig. 3a)
+    # the paper's 10-bit quantized nodes (Fig. 3b) and FP32 nodes (Fig. 3a), walked
+    # by 16 particles per warp (the default mapping reads no nodes)
     node_formats = {}
-    fmt_now = nl.get_option(_lib.QBVH_OPT_NODE_FORMAT)
+    fmt_now, wp_now = nl.get_option(_lib.QBVH_OPT_NODE_FORMAT), nl.get_option(_lib.QBVH_OPT_WARP_PARTICLES)
+    nl.set_option(_lib.QBVH_OPT_WARP_PARTICLES, 16)
     for fmt, name in ((0, "quantized_10bit_16B"), (1, "fp32_32B"), (2, "quantized_21bit_32B")):
         nl.set_option(_lib.QBVH_OPT_NODE_FORMAT, fmt)
         for _ in range(3):
@@ -365,6 +369,7 @@ def run_ours(args):
         node_formats[name] = {"build_ms": float(np.median(tb)), "query_ms": float(np.median(tq)),
                               "nlist_particles_per_s": n / ((float(np.median(tb)) + float(np.median(tq))) * 1e-3)}
     nl.set_option(_lib.QBVH_OPT_NODE_FORMAT, fmt_now)
+    nl.set_option(_lib.QBVH_OPT_WARP_PARTICLES, wp_now)
     step(pos4)
     torch.cuda.synchronize()
 
@@ -434,6 +439,11 @@ def run_ours(args):
         opts_now = autotune.option_names({k: nl.get_option(k) for k in autotune.OPTION_SPACE})
         q_only = bytes_q / (float(t_query.mean()) * 1e-3) / 1e9
         nlist_ms = float(s_build.mean()) + float(t_query.mean())
+        wide = (nl.get_option(_lib.QBVH_OPT_TRAVERSAL) == 1 and
+                nl.get_option(_lib.QBVH_OPT_WARP_PARTICLES) == 32)
+        kname_query = ("wide_query_kernel" if wide else
+                       "query_warp_kernel" if nl.get_option(_lib.QBVH_OPT_TRAVERSAL) == 1 else
+                       "query_thread_kernel") + " (traversal + exact leaf test + list write)"
         if fused:
             # the traversal also reads nothing more and writes the forces (12 B per particle)
             bytes_k = bytes_q + 12 * n
@@ -443,7 +453,7 @@ def run_ours(args):
         else:
             bytes_k = bytes_q
             achieved = q_only
-            kname = "query_warp_kernel (traversal + exact leaf test + list write)"
+            kname = kname_query
         step_alg = (bytes_q + 12 * n) / (float(t_step.mean()) * 1e-3) / 1e9
         value = world * n * args.steps / (total_ms * 1e-3)
         out = {
@@ -489,7 +499,7 @@ def run_ours(args):
                 "peak_source": peak_src,
                 "alg_bytes_per_launch": bytes_k,
                 "step_frac": step_alg / hbm,
-                "query_only": {"kernel": "query_warp_kernel (traversal + exact leaf test + list write)",
+                "query_only": {"kernel": kname_query,
                                "query_ms": float(t_query.mean()), "alg_bytes_per_launch": bytes_q,
                                "achieved": q_only, "frac": q_only / hbm,
                                "traffic": _profiled_traffic(dict(opts_now, fused_lj=0), n),
@@ -501,7 +511,8 @@ def run_ours(args):
                     "steps": e2e_steps, "ms_per_step": e2e_ms / e2e_steps,
                     "copies": "second stream, double-buffered: step k's D2H and step k+1's H2D overlap step k",
                     "l2": "not flushed; every step writes and reads its 1 GB list, larger than L2"},
-            "gpu_launches": args.steps * (KERNELS_PER_STEP_FUSED if fused else KERNELS_PER_STEP),
+            "gpu_launches": args.steps * (KERNELS_PER_STEP_FUSED if fused else
+                                          KERNELS_PER_STEP + (KERNELS_SPREAD if wide else 0)),
             "autotune": {"evaluations": tune_evals, "chosen": autotune.option_names(
                 {k: nl.get_option(k) for k in autotune.OPTION_SPACE})},
             "clocks": clocks,
@@ -570,7 +581,7 @@ def run_batched(args, local):
         g.replay()
 
     space = {k: autotune.OPTION_SPACE[k] for k in (_lib.QBVH_OPT_BUNDLE, _lib.QBVH_OPT_NODE_FORMAT,
-                                                   _lib.QBVH_OPT_QUERY_BLOCK, _lib.QBVH_OPT_PERSISTENT)}
+                                                   _lib.QBVH_OPT_QUERY_BLOCK)}
     space[_lib.QBVH_OPT_WARP_PARTICLES] = [32, 16, 8]
     best, _, _ = autotune.tune(graph_step, space=space, reps=3, warmup=1, sweeps=1)
     g = runners[tuple(sorted(best.items()))]
@@ -1037,7 +1048,7 @@ def main():
     ap.add_argument("--node-format", type=int, default=-1,
                     help="0: 10-bit quantized nodes, 1: FP32 nodes (-1: library default)")
     ap.add_argument("--persistent", type=int, default=-1,
-                    help="traversal warps take packets from a queue (1) or one packet per warp (0); -1: autotuned")
+                    help="accepted without effect, as QBVH_OPT_PERSISTENT is")
     ap.add_argument("--fused-lj", type=int, default=-1,
                     help="LJ terms inside the traversal (1) or a separate list pass (0); -1: autotuned")
     ap.add_argument("--traversal", type=int, default=-1,

@@ -4,10 +4,11 @@ The paper lets runtime autotuners pick the kernel launch parameters during
 warm-up and then freezes them (Sec. 4).  Here the tuned options are the
 subtree-collapse size, the node format (10-bit or 21-bit quantized, or FP32
 bounds: the bit width of the quantization, Sec. 2.2), the
-traversal mapping (thread or warp per particle), the traversal block size,
-whether traversal warps take packets from a queue, and the lanes per particle
-of the LJ pass; where every type pair has the same
+traversal mapping (thread or warp per particle), the traversal block size and
+the lanes per particle of the LJ pass; where every type pair has the same
 list radius a caller may add one tree per system instead of one per type.
+The default mapping walks 32-wide boxes and reads neither the subtrees nor the
+nodes of the binary tree, so the mappings come first in the search.
 The search is coordinate descent:
 each option in turn is swept with the others held at the best values so far,
 for a fixed number of sweeps; every candidate is timed with CUDA events on
@@ -25,13 +26,12 @@ from . import _lib
 __all__ = ["OPTION_SPACE", "OPTIONAL_SPACE", "DEFAULTS", "tune", "time_step", "option_names"]
 
 OPTION_SPACE = {
-    _lib.QBVH_OPT_BUNDLE: [8, 16, 32, 64],
-    _lib.QBVH_OPT_NODE_FORMAT: [0, 1, 2],
     _lib.QBVH_OPT_TRAVERSAL: [1, 0],
     _lib.QBVH_OPT_WARP_PARTICLES: [32, 16, 8, 4, 1],
+    _lib.QBVH_OPT_BUNDLE: [8, 16, 32, 64],
+    _lib.QBVH_OPT_NODE_FORMAT: [0, 1, 2],
     _lib.QBVH_OPT_QUERY_BLOCK: [64, 128, 256],
     _lib.QBVH_OPT_LJ_LANES: [1, 2, 4, 8],
-    _lib.QBVH_OPT_PERSISTENT: [0, 1],
 }
 
 # options a caller adds to the search where they apply: one tree per system
@@ -51,7 +51,6 @@ DEFAULTS = {
     _lib.QBVH_OPT_LJ_LANES: 2,
     _lib.QBVH_OPT_TYPE_TREES: 1,
     _lib.QBVH_OPT_FUSED_LJ: 0,
-    _lib.QBVH_OPT_PERSISTENT: 0,
 }
 
 _NAMES = {
