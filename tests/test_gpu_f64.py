@@ -187,3 +187,35 @@ def test_spinodal_like_1m_fp64():
     idx = np.sort(np.random.default_rng(1).choice(s.n, 8192, replace=False))
     assert_same_lists(rg, cg, ro, co, idx=idx)
     nl.close()
+
+
+@pytest.mark.parametrize("n,n_types", [(1, 1), (33, 2), (5000, 1), (70001, 3)])
+def test_tree_of_double_precision_data(n, n_types):
+    """Exact lists of double-precision data read no nodes, but the tree is there for
+    qbvh_tree_get: positions that are FP32 numbers give the single-precision build's
+    nodes and order, word for word."""
+    import torch
+
+    from paper_1901_08088_gb300 import NeighborList
+
+    rng = np.random.default_rng(n)
+    L = np.float32(max(4.0, (n / 0.7) ** (1 / 3)))
+    x = rng.uniform(0, L, (n, 3)).astype(np.float32)
+    x[x >= L] = 0
+    t = rng.integers(0, n_types, n).astype(np.int32)
+    trees = []
+    for f64 in (False, True):
+        nl = NeighborList(0)
+        if f64:
+            nl.build_f64(torch.from_numpy(workloads.pack_double4(x.astype(np.float64), t)).cuda(), float(L), n_types)
+        else:
+            nl.build(torch.from_numpy(workloads.pack_float4(x, t)).cuda(), float(L), n_types)
+        torch.cuda.synchronize()
+        trees.append({k: v.cpu().numpy().copy() for k, v in nl.tree().items()})
+        nl.close()
+    for k in ("order", "seg_start", "frames"):
+        assert np.array_equal(trees[0][k], trees[1][k]), k
+    inner = np.ones(n, bool)   # a tree of m leaves has m - 1 nodes
+    inner[trees[0]["seg_start"][1:][np.diff(trees[0]["seg_start"]) > 0] - 1] = False
+    assert np.array_equal(trees[0]["nodes"][inner], trees[1]["nodes"][inner])
+    assert np.array_equal(trees[0]["leaves"][:, :3], trees[1]["leaves"][:, :3])

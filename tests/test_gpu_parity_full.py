@@ -94,3 +94,36 @@ def test_config5_every_row_of_every_system(type_trees):
         ro = np.where(np.arange(CAP)[None, :] < co[:, None], ro + a, ro)
         assert_same_lists_chunked(rows[a:b], cg[a:b], ro, co)
     nl.close()
+
+
+@pytest.mark.parametrize("fmt,bundle,traversal,wp,fused", [
+    (2, 64, 1, 16, 0), (2, 64, 1, 8, 0), (2, 32, 0, 32, 0), (1, 64, 0, 32, 0),
+    (0, 64, 1, 32, 1), (1, 64, 1, 32, 1), (2, 64, 1, 32, 1),
+], ids=["21bit_two_lanes", "21bit_four_lanes", "21bit_thread", "fp32_thread", "10bit_fused", "fp32_fused",
+        "21bit_fused"])
+def test_all_2m_rows_through_the_nodes_of_each_format(fluid_2m, fmt, bundle, traversal, wp, fused):
+    """The mappings that walk the binary tree, over each format's node words."""
+    import torch
+
+    from paper_1901_08088_gb300 import NeighborList, _lib
+
+    s, ro, co = fluid_2m
+    nl = NeighborList(0)
+    nl.set_option(_lib.QBVH_OPT_BUNDLE, bundle)
+    nl.set_option(_lib.QBVH_OPT_NODE_FORMAT, fmt)
+    nl.set_option(_lib.QBVH_OPT_TRAVERSAL, traversal)
+    nl.set_option(_lib.QBVH_OPT_WARP_PARTICLES, wp)
+    nl.set_option(_lib.QBVH_OPT_FUSED_LJ, fused)
+    pos4 = torch.from_numpy(workloads.pack_float4(s.pos, s.types)).cuda()
+    nl.build(pos4, s.L)
+    if fused:
+        one = torch.ones((1, 1), device="cuda")
+        U = torch.empty(1, device="cuda", dtype=torch.float64)
+        nl.query_lj_async(pos4, s.r_list, CAP, one, one, np.full((1, 1), 3.0, np.float32), U=U)
+        torch.cuda.synchronize()
+        assert nl.query_status()[0] == _lib.QBVH_OK
+    else:
+        nl.query(s.r_list, cap=CAP)
+    rows, counts = nl.neighbors()
+    assert_same_lists_chunked(rows, counts.cpu().numpy(), ro, co)
+    nl.close()
