@@ -24,12 +24,12 @@ constexpr int kLJBlock = 128;
 
 // Measured before -> here (forward and FP64 sums, microseconds): N = 30,011 97 ->
 // 33; 131,072 with r = 1.12 40 -> 27; 262,144 124 -> 100; the L = 100 mixture 324 ->
-// 141; liquid/vapor 1,000,000 255 -> 226; two-type gradients 32 x 65,536 773 -> 552;
+// 141; liquid/vapor 1,000,000 255 -> 226; two-type gradients 32 x 65,536 773 -> 555;
 // 256 uneven systems 477 -> 426; 2,097,152 646 -> 599.
 //
 // Register cap: 7 blocks of 128 threads.  One type, N = 2,097,152, 10 / 9 / 8 / 7
 // blocks: 711 / 618 / 599 / 597 us; two types with gradients, 32 x 65,536, 9 / 8 / 7
-// blocks / no cap: 580 / 568 / 551 / 683 us.
+// blocks / no cap: 580 / 568 / 551 / 683 us (lanes' gradient sums in FP32 then).
 #ifndef QBVH_LJ_MIN_BLOCKS
 #define QBVH_LJ_MIN_BLOCKS 7
 #endif
@@ -307,7 +307,9 @@ __global__ void pack_kernel(const float *xyz, const int *types, int n, float4 *o
 }  // namespace
 
 // Particles per block: 256, halved down to one round while the grid would hold
-// fewer than 36 blocks per SM (four times what stays resident).
+// fewer than 36 blocks per SM.  (Seven stay resident.  18 / 36 / 72 blocks per SM,
+// microseconds: one type, N = 131,072 53 / 52 / 55, 1,000,000 220 / 212 / 221; two types
+// with gradients, 1,000,000 302 / 300 / 321, 2,097,152 577 / 577 / 588.)
 int lj_particles_per_block(int n, int tpp)
 {
     const int round = kLJBlock / (tpp == 0 ? 8 : tpp);

@@ -687,9 +687,8 @@ __device__ __forceinline__ bool cube_overlap(unsigned nlo, unsigned nhi, const L
 #ifndef QBVH_LOOP_COST
 #define QBVH_LOOP_COST 14
 #endif
-// the walks that filter bundles: exact lists with one particle per lane (FP32
-// or double-precision data), or of FP32 data with 2 or 4 lanes per particle
-// (those share a row through the staging ring, so they need it, and the
+// the walks that filter bundles: exact lists with one particle per lane (reached
+// with the LJ terms), or with 2 or 4 lanes per particle (those share a row through the staging ring, so they need it, and the
 // one-launch walk)
 #ifndef QBVH_MULTI_LANE_FILTER
 #define QBVH_MULTI_LANE_FILTER 1

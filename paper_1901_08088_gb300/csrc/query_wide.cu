@@ -34,7 +34,7 @@
 //      u_j = fl(x_j - nL) as staged, the sign of t shifted into a 32-bit mask (5
 //      to 6 instructions per survivor).  Survivors of different images share
 //      a group.  t is not the list's decision; it decides outside a band around
-//      0 and a group with some |t| inside the band is decided again by the pinned
+//      0, and a group's pairs with |t| inside the band are decided by the pinned
 //      expression on the leaves.  The band, with u = 2^-24:
 //      zero image: u_j = x_j, the components are the pinned ones, d2 and t differ
 //      by at most 6.1 u r^2 where d2 is near r^2; band 2^-20 r^2 (16 u r^2).  Far
@@ -58,11 +58,11 @@
 // header bounds by the padded radius; the test keeps every box and leaf that
 // some lane's exact test could accept.
 //
-// Measured (query launch alone, rope walk before -> here, microseconds): N = 1000
-// 181 -> 20; 30,011 256 -> 58; 131,072 with r = 1.42 190 -> 65; 131,072 in double
-// precision 339 -> 130; 262,144 327 -> 159; the L = 100 mixture 576 -> 248; liquid/
-// vapor 1,000,000 646 -> 393; 32 x 65,536 1523 -> 1028; 256 uneven systems 1904 ->
-// 1230; 2,097,152 1242 -> 953.  Bound by instruction issue and shared memory
+// Measured (whole query, rope walk before -> here, microseconds): N = 1000 181 -> 20;
+// 30,011 256 -> 61; 131,072 with r = 1.42 190 -> 67; 131,072 in double precision 339
+// -> 130; 262,144 327 -> 161; the L = 100 mixture 576 -> 251; liquid/vapor 1,000,000
+// 646 -> 399; 32 x 65,536 1523 -> 1029; 256 uneven systems 1904 -> 1236; 2,097,152
+// 1242 -> 959.  Bound by instruction issue and shared memory
 // together (N = 262,144: 62% of the issue rate, 58% of the L1 data pipe); leaving
 // parts out at N = 2,097,152 put 39% of the time in writing the rows, 25% in the
 // group tests, 20% in the chunks' filter, 16% in boxes and set-up.  One code path
@@ -793,11 +793,13 @@ void launch_lanes(const QueryArgs &a, int lanes, int extra, cudaStream_t s)
 
 // Lanes per particle by the number of particles.  Few particles leave most of
 // the GPU idle with 32 of them per warp, and a packet's walk is a serial chain:
-// with 4 lanes per particle a warp has 8 particles, with 32 one.  Measured
-// (microseconds, 32 / 4 / 1 lanes): N = 4096, density 0.6: 22 / 36 / -;
-// N = 14,503 with r = 1.42: 32 / 33 / -; N = 30,011, density 0.7: 68 / 58 / 98;
-// N = 131,072 with r = 1.42: - / 86 / 63 (the 32- and 4-lane figures at the crossings
-// are from the same kernels before their groups shared images).
+// with 4 lanes per particle a warp has 8 particles, with 32 one.  Measured, whole
+// query with its launches (microseconds, 32 / 4 / 1 lanes), density 0.8, radius 3.3: N =
+// 4096 35 / 54 / 64; 8000 46 / 66 / 89; 14,503 58 / 68 / 80; 30,011 83 / 82 / 90; 45,000
+// 111 / 110 / 98; 60,000 137 / 123 / 107.  Radius 1.42: 14,503 37 / 44 / 55; 30,011 49 /
+// 47 / 54; 45,000 63 / 60 / 59; 60,000 81 / 66 / 62; 131,072 135 / 92 / 78.  (Both
+// lines lie on the sides where these figures cross over: 30,000 and 40,000 would be
+// closer, by up to 20 us at 8000 to 14,503 and 15 at 45,000 to 60,000.)
 static int wide_lanes(int n)
 {
     return n < 8000 ? 32 : (n < 60000 ? 4 : 1);
