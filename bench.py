@@ -103,12 +103,17 @@ class ClockSampler:
 
 
 # DRAM bytes (read + write) and warp instructions executed of one traversal launch at
-# N = 2,097,152, measured with ncu (profiles/query_warp_kernel_lj_n2097152.md) for the
+# N = 2,097,152, measured with ncu (profiles/wide_query_and_lj_n262144.md) for the
 # options of each entry and the traversal sources whose SHA-256 prefix is given; any
 # other source or options report null.
 PROFILED_TRAFFIC = {
-    "source_sha256": "",   # the 32-wide walk has not been profiled at this size yet
-    "entries": [],
+    "source_sha256": "c9bac999f9204346",
+    "entries": [
+        {"options": {"traversal": 1, "warp_particles": 32, "query_block": 64, "fused_lj": 0},
+         "bytes": 1_088_194_304, "warp_inst": 796_368_789},
+        {"options": {"traversal": 1, "warp_particles": 32, "query_block": 128, "fused_lj": 0},
+         "bytes": 1_087_931_136, "warp_inst": 796_368_861},
+    ],
 }
 # kernels of one timed step: build = prepare, Morton (+ sort histograms), segment
 # scan, 4 onesweep passes (30-bit keys, 8-bit digits), Karras, fit; query = 1
