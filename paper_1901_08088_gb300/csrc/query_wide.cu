@@ -554,18 +554,19 @@ __device__ __forceinline__ void sparse_walks(const QueryArgs &a)
 // ---- spread packets --------------------------------------------------------
 // The boxes around far-apart particles (a dilute type among a dense one, vapor around
 // a droplet) cover most of the system, and the packet's warp would test most of its
-// leaves, alone and long after the others.  Spread is a run of 32 leaves whose boxes
-// (box1[run], grown by the radius) cover more than kSpreadVolume times what the cubes
-// around 32 separate spheres do and reach more than kSpreadChunks chunks of leaves
-// under the zero image: a gas stays with its packets, which find little.
-// spread_kernel marks these runs and walks their particles one per warp; the packets'
-// walk passes over them.  The rows are the same either way.
+// leaves, alone and long after the others.  Spread is a run of 32 leaves that holds
+// particles whose boxes, grown by the radius, cover more than kSpreadVolume times
+// what the cubes around 32 separate spheres do and reach more than kSpreadChunks
+// chunks of leaves under the zero image: a gas stays with its packets, which find
+// little.  spread_kernel marks these runs and walks their particles one per warp; the
+// packets' walk passes over them.  The rows are the same either way.
 //
 // Query, milliseconds, walk of the binary tree / packets alone / this: 64 particles of
 // a second type among 2,000,000 in double precision 5.1 / 28.9 / 1.9; four types of 64
 // among 2,000,000 of a fifth 4.1 / 27.2 / 1.7; four batched systems of 250,000 with 32
 // each 3.3 / 5.9 / 0.85; a droplet of 1,000,000 with 100,000 vapor particles in a box
-// of 4000, radius 1.2, 1.07 / 1.61 / 0.35.  It costs 2 to 4 us per query (N = 30,011 58 ->
+// of 4000, radius 1.2, 1.07 / 1.61 / 0.34; 31 particles listed only against 1,000,000 of
+// another type in double precision 3.0 / 20.3 / 0.11.  It costs 2 to 4 us per query (N = 30,011 58 ->
 // 61, 131,072 with r = 1.42 65 -> 67, 2,097,152 953 -> 959), and a gas of 1,000,000 at
 // density 0.0005 the counting of its chunks, 119 -> 167 us (binary tree 224).
 //
@@ -599,15 +600,34 @@ __device__ __forceinline__ int seg_of_leaf(const QueryArgs &a, int s)
     return a.wide_keys ? seg_of_sorted<true>(a, s) : seg_of_sorted<false>(a, s);
 }
 
-__device__ __forceinline__ Box box_of_lane(const Box &b, int src)
+__device__ __forceinline__ unsigned code_of_leaf(const QueryArgs &a, int s)   // 30-bit Z-order code
 {
-    return Box{__shfl_sync(FULL, b.lx, src), __shfl_sync(FULL, b.ly, src), __shfl_sync(FULL, b.lz, src),
-               __shfl_sync(FULL, b.hx, src), __shfl_sync(FULL, b.hy, src), __shfl_sync(FULL, b.hz, src)};
+    return QBVH_QMASK & (a.wide_keys ? (unsigned)__ldg(reinterpret_cast<const unsigned long long *>(a.keys_sorted) + s)
+                                     : __ldg(reinterpret_cast<const unsigned *>(a.keys_sorted) + s));
+}
+
+// The side of the highest cell boundary inside the particles of the lanes in `part`:
+// the top bit in which their first and last codes differ.
+__device__ __forceinline__ bool split_side_of(unsigned code, bool part)
+{
+    const unsigned who = __ballot_sync(FULL, part);
+    const unsigned x = __shfl_sync(FULL, code, __ffs(who) - 1) ^ __shfl_sync(FULL, code, 31 - __clz((int)who));
+    return x != 0u && ((code >> (31 - __clz((int)x))) & 1u);
+}
+
+__device__ __forceinline__ bool spread_volume(const Box &a, const Box &b, bool two, float rs)
+{
+    const float d = 2.f * rs;
+    return grown_volume(a, d) + (two ? grown_volume(b, d) : 0.f) > kSpreadVolume * 32.f * d * d * d;
 }
 
 // Comes before the packets' walk.  A block takes every gridDim.x-th run, `runs` per
 // warp (spread ones lie side by side), and shares the particles of the spread ones it
-// finds among its warps.
+// finds among its warps.  A lane compares its run's volume with the smallest sphere
+// of the list; for the runs that this leaves, the warp tries every tree that has
+// particles in the run, with those particles' boxes and that tree's radii (a few
+// particles of a dilute type may follow the last ones of a type that has no list of
+// its own).
 template <bool F64>
 __global__ void __launch_bounds__(256, 4) spread_kernel(const __grid_constant__ QueryArgs a, int runs)
 {
@@ -618,37 +638,50 @@ __global__ void __launch_bounds__(256, 4) spread_kernel(const __grid_constant__ 
     const int lane = threadIdx.x & 31, T = a.n_types;
     const long long run = ((threadIdx.x >> 5) * runs + lane) * (long long)gridDim.x + blockIdx.x;
     bool wide = false;
-    int seg = 0;
-    Packet p{};
     if (lane < runs && 32 * run < a.n) {
-        seg = seg_of_leaf(a, 32 * (int)run);   // of the run's first particle
-        const int ta = seg % T;
-        float rs = 0.f;
-        for (int tb = 0; tb < T; ++tb) rs = fmaxf(rs, a.r_list[ta * T + tb] > 0.f ? a.rs[ta * T + tb] : 0.f);
+        float rs = __int_as_float(0x7F800000);
+        for (int k = 0; k < T * T; ++k)
+            if (a.r_list[k] > 0.f) rs = fminf(rs, a.rs[k]);
         float4 b[4];
         node32_ld(a.box1 + 4 * run, b[0], b[1]);
         node32_ld(a.box1 + 4 * run + 2, b[2], b[3]);
-        p.a = Box{b[0].x, b[0].y, b[0].z, b[0].w, b[1].x, b[1].y};
-        p.b = Box{b[2].x, b[2].y, b[2].z, b[2].w, b[3].x, b[3].y};
-        const float d = 2.f * rs;
-        // (an empty side has lower corners of +inf; a sparse tree has its own walk)
-        wide = grown_volume(p.a, d) + (p.b.lx <= p.b.hx ? grown_volume(p.b, d) : 0.f) > kSpreadVolume * 32.f * d * d * d &&
-               !(!F64 && a.sparse_blocks > 0 && sparse_tree(a, seg));
+        // (an empty side has lower corners of +inf)
+        wide = spread_volume(Box{b[0].x, b[0].y, b[0].z, b[0].w, b[1].x, b[1].y},
+                             Box{b[2].x, b[2].y, b[2].z, b[2].w, b[3].x, b[3].y}, b[2].x <= b[2].w, rs);
     }
     bool mark = false;
     unsigned todo = __ballot_sync(FULL, wide);
     while (todo) {
         const int src = __ffs(todo) - 1;
         todo &= todo - 1u;
-        const int sg = __shfl_sync(FULL, seg, src), sys = sg / T, ta = sg - sys * T;
-        const Packet q{box_of_lane(p.a, src), box_of_lane(p.b, src), true};
-        int n = 0;
-        for (int tb = 0; tb < T && n <= kSpreadChunks; ++tb) {
-            const SegInfo &g = a.seg[sys * T + tb];
-            if (a.r_list[ta * T + tb] > 0.f && g.count > 0)
-                n = chunks_reached(a, g.start, g.start + g.count - 1, q, a.rs2[ta * T + tb], n);
+        const int s = 32 * (int)__shfl_sync(FULL, run, src) + lane;
+        const int seg = s < a.n ? seg_of_leaf(a, s) : -1;
+        const unsigned code = s < a.n ? code_of_leaf(a, s) : 0u;
+        const float4 me = __ldg(a.leaves + min(s, a.n - 1));
+        Query c{};
+        c.xi = me.x;
+        c.yi = me.y;
+        c.zi = me.z;
+        bool found = false;
+        unsigned rest = __ballot_sync(FULL, seg >= 0);
+        while (rest && !found) {
+            const int sg = __shfl_sync(FULL, seg, __ffs(rest) - 1), sys = sg / T, ta = sg - sys * T;
+            const bool part = seg == sg;
+            rest &= ~__ballot_sync(FULL, part);
+            // (a sparse tree has its own walk)
+            if (!F64 && a.sparse_blocks > 0 && sparse_tree(a, sg)) continue;
+            int n = 0;
+            for (int tb = 0; tb < T && n <= kSpreadChunks; ++tb) {
+                const SegInfo &g = a.seg[sys * T + tb];
+                const float rs = a.rs[ta * T + tb];
+                if (!(a.r_list[ta * T + tb] > 0.f) || g.count == 0) continue;
+                const Packet q = make_packet(c, part, split_side_of(code, part), rs);
+                if (spread_volume(q.a, q.b, q.two, rs))
+                    n = chunks_reached(a, g.start, g.start + g.count - 1, q, a.rs2[ta * T + tb], n);
+            }
+            found = n > kSpreadChunks;
         }
-        if (lane == src) mark = n > kSpreadChunks;
+        if (lane == src) mark = found;
     }
     if (lane < runs && 32 * run < a.n) {
         a.spread[run] = mark;
@@ -708,10 +741,7 @@ __global__ void __launch_bounds__(256, W == 1 && !(ONE && F64) ? 3 : 4) wide_que
     if (ONE && marked) return;
     const float4 me = active ? __ldg(a.leaves + s) : make_float4(0.f, 0.f, 0.f, 0.f);
     const int i = active ? row_index(a, s, me) : 0;
-    unsigned code = 0u;   // 30-bit Z-order code
-    if (active)
-        code = QBVH_QMASK & (a.wide_keys ? (unsigned)__ldg(reinterpret_cast<const unsigned long long *>(a.keys_sorted) + s)
-                                         : __ldg(reinterpret_cast<const unsigned *>(a.keys_sorted) + s));
+    const unsigned code = active ? code_of_leaf(a, s) : 0u;
     Query c;
     c.xi = me.x;
     c.yi = me.y;
@@ -733,11 +763,7 @@ __global__ void __launch_bounds__(256, W == 1 && !(ONE && F64) ? 3 : 4) wide_que
             continue;
         }
         const int sys = ONE ? 0 : seg / T;
-        // the side of the highest cell boundary inside the packet: the top bit
-        // in which its first and last codes differ
-        const unsigned who = __ballot_sync(FULL, part);
-        const unsigned x = __shfl_sync(FULL, code, __ffs(who) - 1) ^ __shfl_sync(FULL, code, 31 - __clz((int)who));
-        const bool side = x != 0u && ((code >> (31 - __clz((int)x))) & 1u);
+        const bool side = split_side_of(code, part);
         walk_trees<F64, W>(a, c, out, st, w, sys, ONE ? 0 : seg - sys * T, T, part, side, (packet * G) >> 5, s & 31,
                            wsub);
     }

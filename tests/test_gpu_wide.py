@@ -169,6 +169,12 @@ def test_spread_packets(n, cap):
           [p[1] for p in parts], np.full((2, 2), 1.9, np.float32), T=2, cap=cap)
     x, L = _droplet(n, 300, n)
     _same(_pos4(x), [0, len(x)], [L], 1.9, cap=cap)
+    # a few particles of each type in the run after the last ones of the dense type,
+    # which has no list of its own
+    x, L, t = _dilute(n, 7, 5, n)
+    r = np.full((5, 5), 1.9, np.float32)
+    r[0, 0] = 0.0
+    _same(_pos4(x, t), [0, n], [L], r, T=5, cap=cap)
 
 
 @pytest.mark.parametrize("n", [7000, 30011, 70003])
@@ -216,6 +222,34 @@ def test_a_dilute_type_costs_little():
         best.append(min(ms))
         nl.close()
     assert best[1] <= 3.0 * best[0]
+
+
+@pytest.mark.parametrize("k", [20, 31, 64])
+def test_cross_list_of_a_few_particles(k):
+    """k particles among 1,000,000 of another type, listed across the types only: less
+    work than the list of the others among themselves (0.6 ms; one packet that tests
+    every leaf took 16 to 20 ms in double precision)."""
+    x, L, t = _dilute(1000000, k, 2, 1)
+    pos4 = _pos4(x, t)
+    best = []
+    for T, own in ((1, True), (5, False)):   # five types: no walk of sparse trees
+        nl = NeighborList()
+        r = np.full((T, T), 3.3, np.float32)
+        if not own:
+            r[0, 0] = 0.0
+        nl.build(pos4 if T > 1 else _pos4(x), L, T).query(r, cap=224)
+        ms = []
+        for _ in range(6):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            nl.query_async(r, 224)
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        assert nl.query_status()[0] == 0
+        best.append(min(ms))
+        nl.close()
+    assert best[1] <= best[0]
 
 
 @pytest.mark.parametrize("n", [700, 5000, 20000, 65000])
