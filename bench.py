@@ -107,12 +107,12 @@ class ClockSampler:
 # options of each entry and the traversal sources whose SHA-256 prefix is given; any
 # other source or options report null.
 PROFILED_TRAFFIC = {
-    "source_sha256": "c9bac999f9204346",
+    "source_sha256": "78a15e0578f922d8",
     "entries": [
         {"options": {"traversal": 1, "warp_particles": 32, "query_block": 64, "fused_lj": 0},
-         "bytes": 1_088_194_304, "warp_inst": 796_368_789},
+         "bytes": 1_087_801_856, "warp_inst": 796_368_781},
         {"options": {"traversal": 1, "warp_particles": 32, "query_block": 128, "fused_lj": 0},
-         "bytes": 1_087_931_136, "warp_inst": 796_368_861},
+         "bytes": 1_087_903_488, "warp_inst": 796_368_773},
     ],
 }
 # kernels of one timed step: build = prepare, Morton (+ sort histograms), segment
